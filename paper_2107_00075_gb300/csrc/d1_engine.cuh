@@ -32,20 +32,21 @@
 // sign in place without disturbing concurrent readers.
 //
 // Work decomposition (no result depends on it):
-//   detect, by |H(v)| (defaults; options mid_degree / hub_degree): up to 64
-//   entries one thread per vertex; up to 16384 one warp per vertex; longer
-//   lists one thread block per vertex.  A loser stops at the step that finds
-//   its conflict.  In round 1 every vertex holds color 1, so v loses exactly
-//   when H(v) is not empty and no list is read.  Losers keep their worklist
-//   entry: they are re-appended by source index (the list counters are the
-//   hottest atomics of the kernel).  Setup cuts long rows into 512-entry
-//   items and push into 128-entry items, one warp each.
+//   detect, by |H(v)| (options mid_degree / hub_degree): two worklists of
+//   vertices whose lists a warp searches together (up to 64 entries, up to
+//   16384), and one block per vertex for longer lists.  A loser stops at the
+//   step that finds its conflict.  In round 1 every vertex holds color 1, so v
+//   loses exactly when H(v) is not empty and no list is read.  Losers keep
+//   their worklist entry: they are re-appended by source index (the list
+//   counters are the hottest atomics of the kernel).  Setup cuts long rows into
+//   512-entry items and push into 128-entry items, one warp each.
 // The round loop runs on the device: a CUDA graph with a conditional WHILE
 // node around {assign, detect, push}; the last block of detect updates the
 // round state and sets the loop condition.  Once the worklist has at most
-// tail_w vertices the remaining rounds run in the core phase: on the
-// subgraph the worklist induces, in one thread-block cluster whose CTAs
-// meet at (bounded) cluster barriers -- the only waits in the engine.
+// mid_w vertices the rounds run in one cooperative launch with grid barriers
+// (the mid loop), and the last ones of a dense core on the subgraph the
+// worklist induces, in one thread-block cluster (the core phase).  Their
+// barriers are the only waits in the engine; they are bounded.
 //
 // Batches: graph g owns global vertices [vtx_off[g], vtx_off[g+1]); ids,
 // the priority hash and degrees are graph-local, so every graph is colored
@@ -88,6 +89,11 @@ struct SingleView {
         d = __ldg(rp + v + 1) - r0;
     }
     __device__ __forceinline__ long long begin(int, int r0) const { return r0; }
+    // first overflow word of v, whose row starts at b: v owns deg/32 + 1 words
+    __device__ __forceinline__ long long bm(int v, long long b) const { return (b >> 5) + v; }
+    // the degree in v's priority, from its row length d
+    __device__ __forceinline__ int degree(int, int d) const { return d; }
+    static constexpr bool kSetup = true;   // the engine builds the lists from the rows
 };
 
 // A batch: graph-local row_ptr blocks (n_g + 1 entries each) and graph-local
@@ -115,35 +121,87 @@ struct BatchView {
     __device__ __forceinline__ long long begin(int g, int r0) const {
         return __ldg(nnz_off + g) + r0;
     }
+    __device__ __forceinline__ long long bm(int v, long long b) const { return (b >> 5) + v; }
+    __device__ __forceinline__ int degree(int, int d) const { return d; }
+    static constexpr bool kSetup = true;
+};
+
+// A conflict graph given by lists the caller has built (distance-2 and
+// partial distance-2, net.cu): v's row is ci[beg .. beg + len), the vertices
+// with priority over v first, so the rows are the priority lists as well.
+// The rows may lie in any order.
+struct ListView {
+    const int2* rows;   // {beg, len} per vertex
+    const int* ci;
+    const int* r_ptr;   // the degree in v's priority is r_ptr[v + 1] - r_ptr[v]
+    int bm_words;       // overflow words per vertex
+    __device__ __forceinline__ int graph(int) const { return 0; }
+    __device__ __forceinline__ int base(int) const { return 0; }
+    __device__ __forceinline__ void row(int v, int, long long& b, int& d) const {
+        const int2 x = __ldg(rows + v);
+        b = x.x;
+        d = x.y;
+    }
+    __device__ __forceinline__ int nbr(long long e, int) const { return __ldg(ci + e); }
+    __device__ __forceinline__ long long begin(int, int r0) const { return r0; }
+    __device__ __forceinline__ long long bm(int v, long long) const {
+        return (long long)v * bm_words;
+    }
+    __device__ __forceinline__ int degree(int v, int) const {
+        return __ldg(r_ptr + v + 1) - __ldg(r_ptr + v);
+    }
+    static constexpr bool kSetup = false;
 };
 
 constexpr int kBuildS = 32;     // setup: degree up to this: one thread
 constexpr int kBuildM = 512;    // setup: degree up to this: one warp
 constexpr int kBuildItem = 512; // setup: adjacency items of this length
 constexpr int kPushItem = 128;  // push: adjacency items of this length
-constexpr int kInlinePush = 32; // S-tier winners up to this degree push inline
+// round-varying priorities: longer lists take a block (R-MAT 18, dynamic degree:
+// 14.0 ms with one warp up to 16,384 entries, 5.2 ms)
+constexpr int kVaryingHub = 1024;
+// winners up to this degree push inline: 32 / 128 / 512 take 73.7 / 58.5 / 58.5 ms
+// for the 4096-graph batch and 3.68 / 3.66 / 4.05 ms for R-MAT 20
+constexpr int kInlinePush = 128;
 
-enum : int { ST_OK = 0, ST_NO_PROGRESS = 1, ST_MAX_ROUNDS = 2, ST_TIMEOUT = 3, ST_BARRIER = 4 };
+enum : int {
+    ST_OK = 0, ST_NO_PROGRESS = 1, ST_MAX_ROUNDS = 2, ST_TIMEOUT = 3, ST_BARRIER = 4,
+    ST_LISTS = 5   // ListView: the lists did not fit their buffer
+};
 
-struct State {
+// What every block of a round's kernel reads, in one place: a block reads it
+// once (see enter()), because thousands of warps reading one line of L2 at the
+// same time wait for one another (10,000 to 20,000 cycles for a handful of
+// fields, more than a small round's work).
+struct Hot {
     int round;        // round being executed (1-based)
     int done;         // 1 once the loop has ended
-    int status;       // ST_*
-    int max_color;
+    int mid;          // 1: the graph loop handed the remaining rounds to the mid loop
+    int tail;         // 1: the mid loop handed the remaining rounds to the core phase
     int ns[2];        // S-tier worklist sizes per parity
     int nm[2];        // M-tier worklist sizes
     int nl[2];        // L-tier worklist sizes
-    int bs, bm, bc;   // setup: vertices (S, M) and items (C) per degree class
     int push_cnt;     // push work items queued this round
+    int max_color;
+    int stop;         // mid loop: round in which the time limit had passed (0: none)
+    __host__ __device__ int count(int p) const { return ns[p] + nm[p] + nl[p]; }
+};
+
+struct State : Hot {
+    int status;       // ST_*
+    int bs, bm, bc;   // setup: vertices (S, M) and items (C) per degree class
     unsigned blocks_done;
-    unsigned l_next;  // dynamic index into the L-tier worklist
-    int tail;         // 1: the graph loop handed the remaining rounds to the core phase
+    int bar_timeout;            // mid loop: a barrier wait gave up
     unsigned long long s_next;  // sum of degrees of the next worklist
     unsigned long long h_next;  // sum of |H(v)| over the next worklist
     unsigned long long h_first; // sum of |H(v)| over all vertices
     unsigned long long t0;      // globaltimer at start
     int core_k;       // core phase: vertices of the induced subgraph
     int core_par;     // core phase: parity whose worklist buffers hold its arrays
+    // mid loop grid barrier, arrivals and generation, a line each: the pollers
+    // of one do not delay the arrivals at the other
+    alignas(128) unsigned bar_count;
+    alignas(128) unsigned bar_gen;
 };
 
 template <class V>
@@ -182,11 +240,68 @@ struct Problem {
     int max_rounds;
     int det_s;
     int det_m;
-    int tail_w;        // hand over to the core phase once the worklist is this small (0: never)
+    int mid_w;         // hand over to the mid loop once the worklist is this small (0: never)
+    int tail_w;        // core phase for worklists up to this size (0: never)
     unsigned bar_polls;   // core loop: barrier polls before giving up
     int slow_block;       // test hook: this core-loop CTA starts late (-1: none)
     unsigned slow_ns;     // ... by this much
 };
+
+// A block's copy of the problem and of the round's counters.  Kernels take
+// the state's address beside the problem's, so both loads start at once.
+template <class V>
+struct Ctx {
+    Problem<V> P;
+    Hot h;
+};
+__device__ __forceinline__ void read_hot(Hot& h, const State* st) {
+    if (threadIdx.x < sizeof(Hot) / 4)
+        reinterpret_cast<int*>(&h)[threadIdx.x] =
+            reinterpret_cast<const volatile int*>(st)[threadIdx.x];
+}
+template <class V>
+__device__ __forceinline__ const Problem<V>& enter(Ctx<V>& c, const Problem<V>* Pp,
+                                                   const State* st) {
+    static_assert(sizeof(Problem<V>) % 4 == 0, "copied by words");
+    read_hot(c.h, st);
+    for (int i = threadIdx.x; i < (int)(sizeof(Problem<V>) / 4); i += blockDim.x)
+        reinterpret_cast<int*>(&c.P)[i] = __ldg(reinterpret_cast<const int*>(Pp) + i);
+    __syncthreads();
+    return c.P;
+}
+
+// Appends entries to the worklists of two tiers, a block's at once: one
+// atomic per block and tier instead of one per warp (the list counters are
+// single addresses that the whole grid hits).  Every thread of the block
+// calls; s_n: 2 x 33 ints of shared memory.
+__device__ __forceinline__ void block_append(bool a, bool b, int4 e, int4* la, int* ca, int4* lb,
+                                             int* cb, int (*s_n)[33]) {
+    const int lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const unsigned ma = __ballot_sync(kFullMask, a), mb = __ballot_sync(kFullMask, b);
+    if (lane == 0) {
+        s_n[0][warp] = __popc(ma);
+        s_n[1][warp] = __popc(mb);
+    }
+    __syncthreads();
+    if (warp < 2) {   // warp 0 places the first tier, warp 1 the second
+        const int x = lane < wpb ? s_n[warp][lane] : 0;
+        int incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFullMask, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int base = 0;
+        if (lane == 31 && incl) base = atomicAdd(warp ? cb : ca, incl);
+        base = __shfl_sync(kFullMask, base, 31);
+        if (lane < wpb) s_n[warp][lane] = base + incl - x;
+    }
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    if (a) la[s_n[0][warp] + __popc(ma & lt)] = e;
+    if (b) lb[s_n[1][warp] + __popc(mb & lt)] = e;
+    __syncthreads();
+}
 
 // key(u) > key(v) for u, v of the same graph (hash of graph-local ids),
 // hashing only when the degree term does not decide.
@@ -199,11 +314,6 @@ __device__ __forceinline__ bool higher(int du, int u, int dv, uint64_t hv, int v
 }
 
 __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; }
-
-
-__device__ __forceinline__ long long bm_offset(long long row_begin, int v) {
-    return (row_begin >> 5) + v;
-}
 
 // Forbid color c for u (a vertex of graph g).  Setting bits of an already
 // colored vertex is harmless (its set is never read again), so colors 1..64
@@ -231,10 +341,10 @@ __device__ __forceinline__ void push_color_live(const Problem<V>& P, int u, int 
     if (c - 1 > du) return;   // u's own first fit never reaches c
     const int b = c - 65;
     if (VARYING && P.prio_mode == 2) {
-        const unsigned old = atomicOr(P.bmx + bm_offset(bu, u) + (b >> 5), 1u << (b & 31));
+        const unsigned old = atomicOr(P.bmx + P.g.bm(u, bu) + (b >> 5), 1u << (b & 31));
         if (!(old & (1u << (b & 31)))) atomicAdd(P.prio + u, 1);
     } else {
-        atomicOr(P.bmx + bm_offset(bu, u) + (b >> 5), 1u << (b & 31));
+        atomicOr(P.bmx + P.g.bm(u, bu) + (b >> 5), 1u << (b & 31));
     }
 }
 template <class V>
@@ -260,18 +370,13 @@ __device__ __forceinline__ void graph_max(int* arr, bool pred, int g, int val) {
 // ---------------------------------------------------------------------------
 template <class V>
 __global__ void d1_classify(const Problem<V>* __restrict__ Pp) {
-    extern __shared__ int smem[];
+    __shared__ int s_n[2][33];
     const Problem<V>& P = *Pp;
     State* st = P.st;
-    const int warp = threadIdx.x >> 5;
-    int4* sm4 = reinterpret_cast<int4*>(smem);
-    WarpAppend4 as = {sm4 + warp * 2 * kAppend4Slots, 0},
-                am = {sm4 + warp * 2 * kAppend4Slots + kAppend4Slots, 0};
     const int n = P.n;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long wbase = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); wbase < n;
-         wbase += stride) {
-        const long long i = wbase + lane_id();
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
+        const long long wbase = base + (threadIdx.x & ~31u), i = wbase + lane_id();
         const bool valid = i < n;
         int d = -1, r0 = 0;
         if (valid) {
@@ -285,7 +390,7 @@ __global__ void d1_classify(const Problem<V>* __restrict__ Pp) {
             P.hlen[v] = 0;
             P.bm0[v] = 0ull;
             if (d >= 64) {
-                unsigned* w = P.bmx + bm_offset(b, v);
+                unsigned* w = P.bmx + P.g.bm(v, b);
                 for (int k = 0; k <= (d >> 5); ++k) w[k] = 0u;
             }
             if (d > kBuildM) {
@@ -295,13 +400,11 @@ __global__ void d1_classify(const Problem<V>* __restrict__ Pp) {
             }
         }
         const unsigned vm = __ballot_sync(kFullMask, valid);
-        if (lane_id() == 0) P.live[wbase >> 5] = vm;   // wbase is a multiple of 32
-        const int4 ent = make_int4((int)i, 0, d, r0);
-        wa4_push(as, valid && d <= kBuildS, ent, P.ws[0], &st->bs);
-        wa4_push(am, valid && d > kBuildS && d <= kBuildM, ent, P.wm[0], &st->bm);
+        // wbase is a multiple of 32 (past n only in the last block's spare warps)
+        if (lane_id() == 0 && vm) P.live[wbase >> 5] = vm;
+        block_append(valid && d <= kBuildS, valid && d > kBuildS && d <= kBuildM,
+                     make_int4((int)i, 0, d, r0), P.ws[0], &st->bs, P.wm[0], &st->bm, s_n);
     }
-    wa4_flush(as, P.ws[0], &st->bs);
-    wa4_flush(am, P.wm[0], &st->bm);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->round = 1;
         st->t0 = global_ns();
@@ -415,55 +518,31 @@ __global__ void __maxnreg__(40) d1_build(const Problem<V>* __restrict__ Pp, int 
     if (lane == 0 && my_h) atomicAdd(&st->h_first, my_h);
 }
 
-// Append v to the worklist of its H-list tier (all 32 lanes call).
-struct TierAppend {
-    WarpAppend4 s, m;
-};
-
-__device__ __forceinline__ TierAppend tier_appender(int* smem) {
-    int4* sm4 = reinterpret_cast<int4*>(smem);
-    const int warp = threadIdx.x >> 5;
-    return TierAppend{{sm4 + warp * 2 * kAppend4Slots, 0},
-                      {sm4 + warp * 2 * kAppend4Slots + kAppend4Slots, 0}};
-}
-
-// e = {v, |H(v)|, deg(v), local row start}
-template <class V>
-__device__ __forceinline__ void tier_push(const Problem<V>& P, TierAppend& a, bool pred, int4 e,
-                                          int p) {
-    State* st = P.st;
-    const int hl = e.y;
-    wa4_push(a.s, pred && hl <= P.det_s, e, P.ws[p], &st->ns[p]);
-    wa4_push(a.m, pred && hl > P.det_s && hl <= P.det_m, e, P.wm[p], &st->nm[p]);
-    if (pred && hl > P.det_m) P.wl[p][atomicAdd(&st->nl[p], 1)] = e;
-}
-
 // ---------------------------------------------------------------------------
 // setup 3: round-1 worklists by |H(v)|
 // ---------------------------------------------------------------------------
 template <class V>
 __global__ void d1_tier(const Problem<V>* __restrict__ Pp) {
-    extern __shared__ int smem[];
+    __shared__ int s_n[2][33];
     const Problem<V>& P = *Pp;
-    TierAppend a = tier_appender(smem);
+    State* st = P.st;
     const int n = P.n;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long wbase = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); wbase < n;
-         wbase += stride) {
-        const long long i = wbase + lane_id();
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
+        const long long i = base + threadIdx.x;
         const bool valid = i < n;
-        int4 e = make_int4((int)i, 0, 0, 0);
+        int4 e = make_int4((int)i, 0, 0, 0);   // {v, |H(v)|, deg(v), local row start}
         if (valid) {
             int r0, d;
             P.g.local_row((int)i, P.g.graph((int)i), r0, d);
             e = make_int4((int)i, P.hlen[i], d, r0);
         }
-        tier_push(P, a, valid, e, 1);
+        block_append(valid && e.y <= P.det_s, valid && e.y > P.det_s && e.y <= P.det_m, e,
+                     P.ws[1], &st->ns[1], P.wm[1], &st->nm[1], s_n);
+        if (valid && e.y > P.det_m) P.wl[1][atomicAdd(&st->nl[1], 1)] = e;
     }
-    wa4_flush(a.s, P.ws[1], &P.st->ns[1]);
-    wa4_flush(a.m, P.wm[1], &P.st->nm[1]);
-    // a graph of at most tail_w vertices runs all its rounds in the core phase
-    if (blockIdx.x == 0 && threadIdx.x == 0 && n <= P.tail_w) P.st->tail = 1;
+    // a graph of at most mid_w vertices runs all its rounds in the mid loop
+    if (blockIdx.x == 0 && threadIdx.x == 0 && n <= P.mid_w) st->mid = 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -472,20 +551,20 @@ __global__ void d1_tier(const Problem<V>* __restrict__ Pp) {
 // First fit for worklist entry e = {v, |H(v)|, deg(v), local row start}.
 // The forbidden set only grows from round to round (committed colors are
 // final), so the first free color never decreases: the scan starts at the
-// previous round's tentative color, -col[v].
+// previous round's tentative color tp = -col[v].  w0: v's first 64 colors,
+// loaded by the caller together with tp (neither waits for the other).
 template <class V>
-__device__ __forceinline__ int first_fit(const Problem<V>& P, int4 e, int tp) {
+__device__ __forceinline__ int first_fit(const Problem<V>& P, int4 e, int tp,
+                                         unsigned long long w0) {
     const int v = e.x;
     int t;
-    unsigned long long w0 = ~0ull;
-    if (tp <= 64) w0 = P.bm0[v];
     if (w0 != ~0ull) {
         t = __ffsll((long long)~w0);
     } else {   // colors 1..64 all taken: deg(v) >= 64, scan the overflow bitmap
         const int g = P.g.graph(v);
         const long long b = P.g.begin(g, e.w);
         const int words = (e.z >> 5) + 1;
-        const unsigned* w = P.bmx + bm_offset(b, v);
+        const unsigned* w = P.bmx + P.g.bm(v, b);
         // four words per step, from the word that holds the previous color
         int k = tp > 64 ? (tp - 65) >> 5 : 0;
         for (;;) {
@@ -517,16 +596,36 @@ __device__ __forceinline__ int first_fit(const Problem<V>& P, int4 e, int tp) {
 }
 
 template <class V>
-__device__ __forceinline__ void assign_phase(const Problem<V>& P) {
-    State* st = P.st;
-    const int cp = *(volatile int*)&st->round & 1;
-    const int n0 = st->ns[cp], n1 = st->nm[cp], n2 = st->nl[cp];
+__device__ __forceinline__ void assign_phase(const Problem<V>& P, const Hot& h) {
+    const int cp = h.round & 1;
+    const int n0 = h.ns[cp], n1 = h.nm[cp], n2 = h.nl[cp];
     const long long total = (long long)n0 + n1 + n2;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        const int4 e = i < n0 ? P.ws[cp][i]
+    // two vertices per thread and step, their loads side by side
+    for (long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < total;
+         i0 += 2 * stride) {
+        int4 e[2];
+        int tp[2];
+        unsigned long long w0[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const long long i = i0 + j * stride;
+            e[j] = make_int4(-1, 0, 0, 0);
+            if (i < total)
+                e[j] = i < n0 ? P.ws[cp][i]
                      : (i < n0 + n1 ? P.wm[cp][i - n0] : P.wl[cp][i - n0 - n1]);
-        P.col[e.x] = -first_fit(P, e, -P.col[e.x]);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            tp[j] = e[j].x >= 0 ? -P.col[e[j].x] : 0;
+            w0[j] = e[j].x >= 0 ? P.bm0[e[j].x] : 0ull;
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (e[j].x >= 0) {
+                const int t = first_fit(P, e[j], tp[j], w0[j]);
+                if (t != tp[j]) P.col[e[j].x] = -t;
+            }
     }
 }
 
@@ -539,10 +638,9 @@ __device__ __forceinline__ void assign_phase(const Problem<V>& P) {
 // depends on timing, so the result is a proper coloring but not a
 // deterministic one; detection is the same snapshot rule as always.
 template <class V>
-__device__ __forceinline__ void assign_async_phase(const Problem<V>& P) {
-    State* st = P.st;
-    const int cp = *(volatile int*)&st->round & 1;
-    const int n0 = st->ns[cp], n1 = st->nm[cp], n2 = st->nl[cp];
+__device__ __forceinline__ void assign_async_phase(const Problem<V>& P, const Hot& h) {
+    const int cp = h.round & 1;
+    const int n0 = h.ns[cp], n1 = h.nm[cp], n2 = h.nl[cp];
     const long long total = (long long)n0 + n1 + n2;
     const int lane = lane_id(), wpb = blockDim.x >> 5;
     const long long gw = (long long)blockIdx.x * wpb + (threadIdx.x >> 5);
@@ -559,7 +657,7 @@ __device__ __forceinline__ void assign_async_phase(const Problem<V>& P) {
             if (w == 0) {
                 f = P.bm0[v];
             } else {   // overflow bitmap words for colors 64w+1 .. 64w+64
-                const unsigned* x = P.bmx + bm_offset(beg, v);
+                const unsigned* x = P.bmx + P.g.bm(v, beg);
                 const int k = 2 * (w - 1), words = (d >> 5) + 1;
                 const unsigned lo = k < words ? x[k] : 0u;
                 const unsigned hi = k + 1 < words ? x[k + 1] : 0u;
@@ -584,17 +682,18 @@ __device__ __forceinline__ void assign_async_phase(const Problem<V>& P) {
 }
 
 template <class V>
-__global__ void d1_assign(const Problem<V>* __restrict__ Pp, cudaGraphConditionalHandle h,
-                          int use_cond) {
-    const Problem<V>& P = *Pp;
+__global__ void d1_assign(const Problem<V>* __restrict__ Pp, State* st,
+                          cudaGraphConditionalHandle h, int use_cond) {
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // The loop continues only if this round's detect says so: should its
         // round control ever not run, the device loop ends instead of spinning.
         if (use_cond) cudaGraphSetConditional(h, 0u);
-        P.st->push_cnt = 0;   // the previous round's push kernel has finished
+        st->push_cnt = 0;   // the previous round's push kernel has finished
     }
-    if (P.async_mode) assign_async_phase(P);
-    else assign_phase(P);
+    if (P.async_mode) assign_async_phase(P, ctx.h);
+    else assign_phase(P, ctx.h);
 }
 
 // ---------------------------------------------------------------------------
@@ -638,26 +737,35 @@ __device__ int round_decide(const Problem<V>& P) {
     st->status = status;
     st->done = done;
     st->blocks_done = 0u;
-    st->l_next = 0u;
-    st->tail = (!done && nxt <= P.tail_w) ? 1 : 0;
+    st->mid = (!done && nxt <= P.mid_w) ? 1 : 0;
     __threadfence();
     return done;
 }
 
 // Round control of the launch-per-round loop: the WHILE node repeats while
-// the coloring is unfinished and the worklist is larger than tail_w; the
-// remaining rounds go to the core phase.
+// the coloring is unfinished and the worklist is larger than mid_w; the
+// remaining rounds go to the mid loop.
 template <class V>
 __device__ void round_control(const Problem<V>& P, cudaGraphConditionalHandle h, int use_cond) {
     const int done = round_decide(P);
-    if (use_cond) cudaGraphSetConditional(h, (done || P.st->tail) ? 0u : 1u);
+    if (use_cond) cudaGraphSetConditional(h, (done || P.st->mid) ? 0u : 1u);
 }
 
-// Queue the push of v's color: ceil(deg / kPushItem) work items.
+// Queue the pushes of the lanes with pred (all 32 call): ceil(deg / kPushItem)
+// work items each, one atomic for all of them.
 template <class V>
-__device__ __forceinline__ void queue_push(const Problem<V>& P, int v, int d) {
-    const int nit = ceil_div(d, kPushItem);
-    const int base = atomicAdd(&P.st->push_cnt, nit);
+__device__ __forceinline__ void queue_push(const Problem<V>& P, bool pred, int v, int d) {
+    if (!__any_sync(kFullMask, pred)) return;
+    const int lane = lane_id(), nit = pred ? ceil_div(d, kPushItem) : 0;
+    int incl = nit;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += y;
+    }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(&P.st->push_cnt, incl);
+    base = __shfl_sync(kFullMask, base, 31) + incl - nit;
     for (int k = 0; k < nit; ++k) P.push_q[base + k] = make_int2(v, k);
 }
 
@@ -698,75 +806,212 @@ __device__ __forceinline__ bool conflict(const Problem<V>& P, int u, int t, MeOf
     else return u >= 0 && abs(P.col[u]) == t;
 }
 
-// Warp-wide: does any of the list entries [b0, min(b0 + 32K, hl)) of v
-// (starting at h) conflict with v's color t?  K ids per lane are loaded,
-// then their K colors, so a step costs two dependent loads whatever K is.
-template <int K, bool DYN, class V>
-__device__ __forceinline__ bool warp_step(const Problem<V>& P, const int* h, int b0, int hl,
-                                          int t, MeOf<DYN> me) {
+// What detection adds up per lane over a round.
+struct RoundSums {
+    int max_color = 0;
+    unsigned long long s = 0ull, h = 0ull;   // degrees and list lengths of the losers
+};
+
+// A step over the rows of the lanes in `open` (not empty): 128 places, the
+// same power of two of consecutive entries for each row, at least four.  Place
+// f = 32 j + lane (j = 0..3) is entry f % per of the row with rank f / per.
+struct Deal {
+    int n, log;   // rows; log2 of the entries per row
+};
+__device__ __forceinline__ Deal deal_rows(unsigned open, unsigned char* slot) {
     const int lane = lane_id();
-    int u[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const int e = b0 + 32 * j + lane;
-        u[j] = e < hl ? __ldg(h + e) : -1;
-    }
-    bool hit = false;
-#pragma unroll
-    for (int j = 0; j < K; ++j) hit |= conflict<DYN>(P, u[j], t, me);
-    return __any_sync(kFullMask, hit);
+    Deal d;
+    d.n = __popc(open);
+    d.log = d.n == 1 ? 7 : __clz(d.n - 1) - 25;
+    __syncwarp();
+    if (open >> lane & 1u) slot[__popc(open & ((1u << lane) - 1u))] = (unsigned char)lane;
+    __syncwarp();
+    return d;
+}
+// The lane whose row has place 32 j + lane (-1: none).
+__device__ __forceinline__ int deal_lane(const Deal& d, const unsigned char* slot, int j) {
+    const int i = (32 * j + (int)lane_id()) >> d.log;
+    return i < d.n ? slot[i] : -1;
+}
+// Does the row with this rank have a place in the four ballots?
+__device__ __forceinline__ bool deal_any(const Deal& d, int rank, const unsigned (&b)[4]) {
+    if (d.log >= 7) return (b[0] | b[1] | b[2] | b[3]) != 0u;
+    if (d.log == 6) return (rank ? b[2] | b[3] : b[0] | b[1]) != 0u;
+    const int from = rank << d.log, j = from >> 5;
+    const unsigned w = j == 0 ? b[0] : j == 1 ? b[1] : j == 2 ? b[2] : b[3];
+    return (w >> (from & 31) & (kFullMask >> (32 - (1 << d.log)))) != 0u;
 }
 
-// Warp-wide: does any of the H-list entries [from, hl) of v (starting at
-// hadj[beg]) currently hold color t?  The steps grow 64, 128, 256, 256, ...
-// entries: most losers meet their conflict in the first step, while a
-// winner, which must read its whole list, needs few dependent steps.
+// One tier's worklist: conflict search, commit, inline push and re-append.
+//
+// A warp takes up to 32 worklist vertices and searches their lists together:
+// in each step the lists still undecided get the same number of places, so a
+// step has up to 128 independent gathers in flight and costs two dependent
+// loads however many lists it serves.  Losers meet their conflict within the
+// first entries (a mean of 2 to 12 on meshes, patterns and R-MAT) and leave;
+// their places go to those that must read on, at last 128 entries per step
+// for one winner.  Consecutive lanes take consecutive entries: an instruction
+// then touches one line per row instead of one per lane, and lines per
+// instruction are what the first-level cache is bound by here (random gathers:
+// 290 G/s measured, one line per SM and cycle).  Small worklists are spread
+// over the warps first (fewer vertices per warp, more places for each).  The
+// winners' pushes deal their rows in the same way.
+//
+// One thread or one warp per vertex with lists read alone, in turn, waited for
+// the longest list of a warp; with the shared counters read once per block
+// (Hot) and appended to once per block, detection of R-MAT 20's first 13
+// rounds went from 0.86 to 0.57 ms, of PD2 4M x 1M's 51 rounds from 9.6 to
+// 4.6 ms, of the 4096-graph batch from 56 to 32 ms.  64 registers (4 blocks
+// per SM) beat 48 with spills (PD2 16.4 against 16.1 ms, R-MAT 20 3.84
+// against 3.66 ms in all).
 template <bool DYN, class V>
-__device__ __forceinline__ bool warp_conflict(const Problem<V>& P, long long beg, int hl, int t,
-                                              int from, MeOf<DYN> me) {
-    const int* h = P.hadj + beg;
-    int b0 = from;
-    if (b0 < hl) {
-        if (warp_step<2, DYN>(P, h, b0, hl, t, me)) return true;
-        b0 += 64;
+__device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* list, int n, int4* next,
+                                            int* next_cnt, IdxAppend& app, unsigned char* slot,
+                                            int r, RoundSums& sum) {
+    const int* __restrict__ ha = P.hadj;
+    int* const col = P.col;
+    const bool batch = P.g_rounds != nullptr, traced = P.trace_cap > 0;
+    // round 1: every vertex holds tentative color 1, so v loses exactly when
+    // H(v) is not empty -- no list needs to be read
+    const bool first = r == 1 && !P.async_mode && !DYN;
+    const int lane = lane_id(), wpb = blockDim.x >> 5;
+    const long long gw = (long long)blockIdx.x * wpb + (threadIdx.x >> 5);
+    const long long nw = (long long)gridDim.x * wpb;
+    int take = 32;   // vertices per warp: the smallest power of two that is one pass
+    while (take > 1 && (take >> 1) * nw >= n) take >>= 1;
+    for (long long i0 = gw * take; i0 < n; i0 += nw * take) {
+        const long long i = i0 + lane;
+        const bool valid = lane < take && i < n;
+        int4 ent = make_int4(0, 0, 0, 0);
+        int g = 0, t = 0;
+        long long beg = 0;
+        MeOf<DYN> me{};
+        if (valid) {
+            ent = list[i];
+            g = P.g.graph(ent.x);
+            beg = P.g.begin(g, ent.w);
+            t = -col[ent.x];
+            if constexpr (DYN) me = round_me(P, ent.x, g);
+        }
+        const int v = ent.x, hl = ent.y, d = ent.z;
+        bool lose = valid && first && hl > 0;
+        int pos = 0;   // entries read of every list still open
+        unsigned open = __ballot_sync(kFullMask, valid && !first && hl > 0);
+        while (open) {   // warp-uniform
+            const Deal deal = deal_rows(open, slot);
+            const int per = 1 << deal.log;
+            int u[4], ut[4];
+            MeOf<DYN> ume[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int src = deal_lane(deal, slot, j), from = src < 0 ? lane : src;
+                const int x = pos + ((32 * j + lane) & (per - 1));
+                const int len = __shfl_sync(kFullMask, hl, from);
+                const long long b = __shfl_sync(kFullMask, beg, from);
+                ut[j] = __shfl_sync(kFullMask, t, from);
+                if constexpr (DYN) {
+                    ume[j].v = __shfl_sync(kFullMask, me.v, from);
+                    ume[j].p = __shfl_sync(kFullMask, me.p, from);
+                    ume[j].base = __shfl_sync(kFullMask, me.base, from);
+                    ume[j].h = __shfl_sync(kFullMask, me.h, from);
+                }
+                u[j] = src >= 0 && x < len ? __ldg(ha + b + x) : -1;
+            }
+            bool hit[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) hit[j] = conflict<DYN>(P, u[j], ut[j], ume[j]);
+            unsigned hits[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) hits[j] = __ballot_sync(kFullMask, hit[j]);
+            bool mine = open >> lane & 1u;
+            if (mine) {
+                lose = deal_any(deal, __popc(open & ((1u << lane) - 1u)), hits);
+                mine = !lose && pos + per < hl;
+            }
+            pos += per;
+            open = __ballot_sync(kFullMask, mine);
+        }
+        const bool win = valid && !lose;
+        if (lose) {
+            sum.s += (unsigned long long)(V::kSetup ? d : traced ? P.g.degree(v, d) : 0);
+            sum.h += (unsigned long long)hl;
+        }
+        if (win) {
+            col[v] = t;
+            atomicAnd(P.live + (v >> 5), ~(1u << (v & 31)));
+            sum.max_color = max(sum.max_color, t);
+        }
+        // with DYN every push is queued: an inline one would change
+        // neighbors' priorities while others still compare them
+        queue_push(P, win && (d > kInlinePush || DYN), v, d);
+        if (batch) {
+            graph_max(P.g_rounds, win, g, r);
+            graph_max(P.g_colors, win, g, t);
+        }
+        if (!DYN) {
+            pos = 0;
+            open = __ballot_sync(kFullMask, win && d <= kInlinePush && d > 0);
+            while (open) {
+                const Deal deal = deal_rows(open, slot);
+                const int per = 1 << deal.log;
+                int u[4], from[4];
+                unsigned lw[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int src = deal_lane(deal, slot, j);
+                    from[j] = src < 0 ? lane : src;
+                    const int x =
+                        __shfl_sync(kFullMask, pos, from[j]) + ((32 * j + lane) & (per - 1));
+                    const int len = __shfl_sync(kFullMask, d, from[j]);
+                    const long long b = __shfl_sync(kFullMask, beg, from[j]);
+                    const int uv = __shfl_sync(kFullMask, v, from[j]);
+                    const int ug = __shfl_sync(kFullMask, g, from[j]);
+                    u[j] = src >= 0 && x < len ? P.g.nbr(b + x, P.g.base(ug)) : -1;
+                    if (u[j] == uv) u[j] = -1;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) lw[j] = u[j] >= 0 ? P.live[u[j] >> 5] : 0u;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int ug = __shfl_sync(kFullMask, g, from[j]);
+                    const int uc = __shfl_sync(kFullMask, t, from[j]);
+                    if ((lw[j] >> (u[j] & 31)) & 1u) push_color_live<false>(P, u[j], ug, uc);
+                }
+                bool mine = open >> lane & 1u;
+                if (mine) {
+                    pos += per;
+                    mine = pos < d;
+                }
+                open = __ballot_sync(kFullMask, mine);
+            }
+        }
+        ia_push(app, lose, (int)i, list, next, next_cnt);
     }
-    if (b0 < hl) {
-        if (warp_step<4, DYN>(P, h, b0, hl, t, me)) return true;
-        b0 += 128;
-    }
-    for (; b0 < hl; b0 += 256)
-        if (warp_step<8, DYN>(P, h, b0, hl, t, me)) return true;
-    return false;
 }
 
 // Detection, commit, compaction and inline push for one round (every block
 // of the grid takes part).  DYN: priorities that change each round -- the
-// lists then hold every neighbor, a neighbor holding v's color must also
-// beat v this round, and every winner's push is queued (an inline push would
-// change neighbors' priorities while others still compare them).
+// lists then hold every neighbor, and a neighbor holding v's color must also
+// beat v this round.
 template <class V, bool DYN>
-__device__ __forceinline__ void detect_phase(const Problem<V>& P, int* smem) {
+__device__ __forceinline__ void detect_phase(const Problem<V>& P, const Hot& hot, int* smem) {
+    __shared__ unsigned char s_slot[32][32];
+    __shared__ int s_n[2][33], s_max;
     State* st = P.st;
-    const int r = *(volatile int*)&st->round;
-    const int cp = r & 1, np = cp ^ 1;
-    const int nS = st->ns[cp], nM = st->nm[cp], nL = st->nl[cp];
+    const int r = hot.round, cp = r & 1, np = cp ^ 1;
+    const int nS = hot.ns[cp], nM = hot.nm[cp], nL = hot.nl[cp];
     const int* __restrict__ ha = P.hadj;
     int* col = P.col;
-    const bool batch = P.g_rounds != nullptr;
     const int lane = lane_id();
     const int warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
-    const int gw = blockIdx.x * wpb + warp, nw = gridDim.x * wpb;
-    int my_max = 0;
-    unsigned long long my_s = 0ull, my_h = 0ull;
+    RoundSums sum;
     // losers keep their entry and tier: appended by source index
     IdxAppend app_s = {smem + warp * 2 * kIdxSlots, 0};
     IdxAppend app_m = {smem + warp * 2 * kIdxSlots + kIdxSlots, 0};
-    // Round 1: every vertex holds tentative color 1, so v loses exactly when
-    // H(v) is not empty -- no list needs to be read.
     const bool first = r == 1 && !P.async_mode && !DYN;
 
-    // --- L tier: one block per vertex (static assignment) ---
+    // --- L tier: one block per vertex (static assignment), four entries per
+    // thread and step ---
     for (int i = blockIdx.x; i < nL; i += gridDim.x) {
         const int4 ent = P.wl[cp][i];
         const int v = ent.x, hl = ent.y, d = ent.z;
@@ -776,174 +1021,87 @@ __device__ __forceinline__ void detect_phase(const Problem<V>& P, int* smem) {
         MeOf<DYN> me{};
         if constexpr (DYN) me = round_me(P, v, g);
         bool lose = first && hl > 0;
-        int nxt = !first && (int)threadIdx.x < hl ? __ldg(ha + beg + threadIdx.x) : -1;
-        for (int b0 = 0; !first && b0 < hl; b0 += blockDim.x) {
-            const int u = nxt;
-            const int e = b0 + blockDim.x + threadIdx.x;
-            nxt = e < hl ? __ldg(ha + beg + e) : -1;
-            if (__syncthreads_or(conflict<DYN>(P, u, t, me))) {
-                lose = true;
-                break;
+        for (int b0 = 0; !first && b0 < hl && !lose; b0 += 4 * blockDim.x) {
+            int u[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int e = b0 + j * blockDim.x + threadIdx.x;
+                u[j] = e < hl ? __ldg(ha + beg + e) : -1;
             }
+            bool hit = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) hit |= conflict<DYN>(P, u[j], t, me);
+            lose = __syncthreads_or(hit);
         }
         if (threadIdx.x == 0) {
             if (lose) {
                 P.wl[np][atomicAdd(&st->nl[np], 1)] = ent;
-                my_s += (unsigned long long)d;
-                my_h += (unsigned long long)hl;
-                if (batch) atomicMax(P.g_rounds + g, r + 1);
+                sum.s += (unsigned long long)P.g.degree(v, d);
+                sum.h += (unsigned long long)hl;
             } else {
                 col[v] = t;
                 atomicAnd(P.live + (v >> 5), ~(1u << (v & 31)));
-                my_max = max(my_max, t);
-                if (batch) atomicMax(P.g_colors + g, t);
-                queue_push(P, v, d);
-            }
-        }
-        __syncthreads();
-    }
-
-    // --- M tier: one warp per vertex.  The next vertex's entry is loaded
-    // while this one's first 32 list colors are gathered, and its own color
-    // and first 32 list ids while this one is committed or appended. ---
-    int4 ent = make_int4(-1, 0, 0, 0);
-    long long beg = 0;
-    int g = 0, t = 0, u0 = -1;
-    if (gw < nM) {
-        ent = P.wm[cp][gw];
-        g = P.g.graph(ent.x);
-        beg = P.g.begin(g, ent.w);
-        t = -col[ent.x];
-        u0 = !first && lane < ent.y ? __ldg(ha + beg + lane) : -1;
-    }
-    for (int i = gw; i < nM; i += nw) {
-        const int v = ent.x, hl = ent.y, d = ent.z;
-        const int in = i + nw;
-        int4 en = make_int4(-1, 0, 0, 0);
-        if (in < nM) en = P.wm[cp][in];
-        MeOf<DYN> me{};
-        if constexpr (DYN) me = round_me(P, v, g);
-        bool lose = first ? hl > 0 : __any_sync(kFullMask, conflict<DYN>(P, u0, t, me));
-        if (!first && !lose && hl > 32) lose = warp_conflict<DYN>(P, beg, hl, t, 32, me);
-        int gn = 0, tn = 0, un = -1;
-        long long bn = 0;
-        if (in < nM) {
-            gn = P.g.graph(en.x);
-            bn = P.g.begin(gn, en.w);
-            tn = -col[en.x];
-            un = !first && lane < en.y ? __ldg(ha + bn + lane) : -1;
-        }
-        if (lane == 0) {
-            if (lose) {
-                my_s += (unsigned long long)d;
-                my_h += (unsigned long long)hl;
-                if (batch) atomicMax(P.g_rounds + g, r + 1);
-            } else {
-                col[v] = t;
-                atomicAnd(P.live + (v >> 5), ~(1u << (v & 31)));
-                my_max = max(my_max, t);
-                if (batch) atomicMax(P.g_colors + g, t);
-                queue_push(P, v, d);
-            }
-        }
-        ia_push(app_m, lose && lane == 0, i, P.wm[cp], P.wm[np], &st->nm[np]);
-        ent = en;
-        beg = bn;
-        g = gn;
-        t = tn;
-        u0 = un;
-    }
-
-    // --- S tier: one thread per vertex ---
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long wbase = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); wbase < nS;
-         wbase += stride) {
-        const long long i = wbase + lane;
-        bool lose = false, win = false;
-        int g = 0, t = 0;
-        int4 ent = make_int4(-1, 0, 0, 0);
-        if (i < nS) {
-            ent = P.ws[cp][i];
-            const int v = ent.x, hl = ent.y, d = ent.z;
-            g = P.g.graph(v);
-            const long long beg = P.g.begin(g, ent.w);
-            t = -col[v];
-            MeOf<DYN> me{};
-            if constexpr (DYN) me = round_me(P, v, g);
-            lose = first && hl > 0;
-            // four list entries, then eight at a time (ids, then their colors)
-            if (!first && hl > 0) {
-                int u[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) u[j] = j < hl ? __ldg(ha + beg + j) : -1;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) lose |= conflict<DYN>(P, u[j], t, me);
-            }
-            for (int e = 4; !first && e < hl && !lose; e += 8) {
-                int u[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) u[j] = e + j < hl ? __ldg(ha + beg + e + j) : -1;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) lose |= conflict<DYN>(P, u[j], t, me);
-            }
-            if (lose) {
-                my_s += (unsigned long long)d;
-                my_h += (unsigned long long)hl;
-            } else {
-                win = true;
-                col[v] = t;
-                atomicAnd(P.live + (v >> 5), ~(1u << (v & 31)));
-                my_max = max(my_max, t);
-                if (d <= kInlinePush && !DYN) {
-                    // four neighbors at a time: ids, then their uncolored
-                    // bits, then the updates
-                    const int base = P.g.base(g);
-                    for (int e0 = 0; e0 < d; e0 += 4) {
-                        int u[4];
-                        unsigned lw[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            u[j] = e0 + j < d ? P.g.nbr(beg + e0 + j, base) : v;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) lw[j] = u[j] != v ? P.live[u[j] >> 5] : 0u;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if ((lw[j] >> (u[j] & 31)) & 1u) push_color_live<false>(P, u[j], g, t);
-                    }
-                } else {
-                    queue_push(P, v, d);
+                sum.max_color = max(sum.max_color, t);
+                if (P.g_rounds != nullptr) {
+                    atomicMax(P.g_rounds + g, r);
+                    atomicMax(P.g_colors + g, t);
                 }
             }
         }
-        if (batch) {
-            graph_max(P.g_rounds, lose, g, r + 1);
-            graph_max(P.g_colors, win, g, t);
-        }
-        ia_push(app_s, lose, (int)i, P.ws[cp], P.ws[np], &st->ns[np]);
+        if (warp == 0) queue_push(P, lane == 0 && !lose, v, d);
+        __syncthreads();
     }
-    ia_flush(app_s, P.ws[cp], P.ws[np], &st->ns[np]);
-    ia_flush(app_m, P.wm[cp], P.wm[np], &st->nm[np]);
 
-    // --- per-warp totals ---
-    my_max = warp_max(my_max);
-    my_s = warp_sum(my_s);
-    my_h = warp_sum(my_h);
+    // --- M tier, then S tier: longer lists first ---
+    detect_tier<DYN>(P, P.wm[cp], nM, P.wm[np], &st->nm[np], app_m, s_slot[warp], r, sum);
+    detect_tier<DYN>(P, P.ws[cp], nS, P.ws[np], &st->ns[np], app_s, s_slot[warp], r, sum);
+
+    // --- what is left in the appenders, and the totals, once per block: one
+    // atomic per warp on the same address would take as long as a small round
+    if (threadIdx.x == 0) s_max = 0;
     if (lane == 0) {
-        if (my_max > 0) atomicMax(&st->max_color, my_max);
-        if (my_s > 0) atomicAdd(&st->s_next, my_s);
-        if (my_h > 0) atomicAdd(&st->h_next, my_h);
+        s_n[0][warp] = app_s.count;
+        s_n[1][warp] = app_m.count;
     }
-
+    __syncthreads();
+    const int my_max = warp_max(sum.max_color);
+    if (lane == 0 && my_max > hot.max_color) atomicMax(&s_max, my_max);
+    if (warp < 2) {
+        const int x = lane < (int)(blockDim.x >> 5) ? s_n[warp][lane] : 0;
+        int incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFullMask, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int base = 0;
+        if (lane == 31 && incl) base = atomicAdd(warp ? &st->nm[np] : &st->ns[np], incl);
+        base = __shfl_sync(kFullMask, base, 31);
+        if (lane < (int)(blockDim.x >> 5)) s_n[warp][lane] = base + incl - x;
+    }
+    __syncthreads();
+    for (int k = lane; k < app_s.count; k += 32)
+        P.ws[np][s_n[0][warp] + k] = P.ws[cp][app_s.buf[k]];
+    for (int k = lane; k < app_m.count; k += 32)
+        P.wm[np][s_n[1][warp] + k] = P.wm[cp][app_m.buf[k]];
+    if (threadIdx.x == 0 && s_max > 0) atomicMax(&st->max_color, s_max);
+    if (P.trace_cap > 0) {
+        const unsigned long long my_s = warp_sum(sum.s), my_h = warp_sum(sum.h);
+        if (lane == 0 && (my_s || my_h)) {
+            atomicAdd(&st->s_next, my_s);
+            atomicAdd(&st->h_next, my_h);
+        }
+    }
 }
 
 template <class V, bool DYN = false>
-__global__ void __maxnreg__(48) d1_detect(const Problem<V>* __restrict__ Pp,
+__global__ void __maxnreg__(64) d1_detect(const Problem<V>* __restrict__ Pp, State* st,
                                           cudaGraphConditionalHandle h, int use_cond) {
     extern __shared__ int smem[];
-    const Problem<V>& P = *Pp;
-    State* st = P.st;
-    if (*(volatile int*)&st->tail) return;   // handed over before round 1
-    detect_phase<V, DYN>(P, smem);
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    if (ctx.h.mid || ctx.h.done) return;   // handed over before round 1, or no lists
+    detect_phase<V, DYN>(P, ctx.h, smem);
 
     // --- last block runs the round control ---
     __shared__ int s_last;
@@ -964,8 +1122,7 @@ __global__ void __maxnreg__(48) d1_detect(const Problem<V>* __restrict__ Pp,
 // push: winners' colors into the forbidden sets of their neighbors
 // ---------------------------------------------------------------------------
 template <class V>
-__device__ __forceinline__ void push_phase(const Problem<V>& P) {
-    const int nq = *(volatile int*)&P.st->push_cnt;
+__device__ __forceinline__ void push_phase(const Problem<V>& P, int nq) {
     const int lane = lane_id(), wpb = blockDim.x >> 5;
     for (int q = blockIdx.x * wpb + (threadIdx.x >> 5); q < nq; q += gridDim.x * wpb) {
         const int2 item = P.push_q[q];
@@ -993,11 +1150,10 @@ __device__ __forceinline__ void push_phase(const Problem<V>& P) {
 // PGC_ASYNC: the next round's worklist vertices start uncolored (0), so that
 // a negative color seen during its first fit is one written in that round.
 template <class V>
-__device__ __forceinline__ void reset_next_worklist(const Problem<V>& P) {
-    const State* st = P.st;
-    if (*(volatile const int*)&st->done) return;
-    const int p = *(volatile const int*)&st->round & 1;
-    const int n0 = st->ns[p], n1 = st->nm[p], n2 = st->nl[p];
+__device__ __forceinline__ void reset_next_worklist(const Problem<V>& P, const Hot& h) {
+    if (h.done) return;
+    const int p = h.round & 1;
+    const int n0 = h.ns[p], n1 = h.nm[p], n2 = h.nl[p];
     const long long total = (long long)n0 + n1 + n2;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -1008,9 +1164,154 @@ __device__ __forceinline__ void reset_next_worklist(const Problem<V>& P) {
 }
 
 template <class V>
-__global__ void d1_push(const Problem<V>* __restrict__ Pp) {
-    push_phase(*Pp);
-    if (Pp->async_mode) reset_next_worklist(*Pp);
+__global__ void d1_push(const Problem<V>* __restrict__ Pp, State* st) {
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    push_phase(P, ctx.h.push_cnt);
+    if (P.async_mode) reset_next_worklist(P, ctx.h);
+}
+
+// ---------------------------------------------------------------------------
+// mid loop: the rounds of a worklist that does not fill the GPU
+// ---------------------------------------------------------------------------
+// Grid-wide barrier for a cooperative launch (all blocks co-resident), then
+// the block's copy of the counters, for round r (the state's own round moves
+// on at the end of the kernel).  A wait that exceeds max_polls polls (2^22:
+// about a second) gives up, records the failure and lets the kernel return
+// with an error.
+__device__ __forceinline__ bool grid_barrier(State* st, Hot& h, unsigned& gen, unsigned max_polls,
+                                             int r) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
+            int ok = 1;
+            unsigned arrived;
+            asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;"
+                         : "=r"(arrived) : "l"(&st->bar_count) : "memory");
+            if (arrived == gridDim.x - 1) {
+                asm volatile("st.relaxed.gpu.u32 [%0], 0;" ::"l"(&st->bar_count) : "memory");
+                asm volatile("red.release.gpu.add.u32 [%0], 1;" ::"l"(&st->bar_gen) : "memory");
+            } else {
+                unsigned polls = 0, now;
+                for (;;) {
+                    asm volatile("ld.acquire.gpu.u32 %0, [%1];"
+                                 : "=r"(now) : "l"(&st->bar_gen) : "memory");
+                    if (now != gen) break;
+                    ++polls;
+                    if (polls > max_polls || ((polls & 15u) == 0u && *(volatile int*)&st->bar_timeout)) {
+                        atomicExch(&st->bar_timeout, 1);
+                        ok = 0;
+                        break;
+                    }
+                    if (polls > 64u) __nanosleep(64);
+                }
+            }
+            s_ok = ok;
+        }
+        __syncwarp();
+        read_hot(h, st);
+        __syncwarp();
+        if (threadIdx.x == 0) h.round = r;
+    }
+    ++gen;
+    __syncthreads();
+    return s_ok != 0;
+}
+
+constexpr int kMidMax = 65536;     // worklists up to this size
+constexpr int kMidThreads = 1024;
+constexpr int kMidShared = 8;      // blocks when several colorings share the GPU (the server) ...
+constexpr int kMidSharedMax = 16384;  // ... and their worklists
+
+// The rounds (assign, detect, push) in one cooperative launch, one block per
+// SM, grid barriers in place of launches.  Every block takes the same round
+// decisions from the counters, so there is no last block to wait for; block 0
+// prepares the next round's counters while everyone assigns.  What bounds a
+// round is its chain of dependent loads (about 10,000 cycles in detection for
+// any worklist) and two or three barriers of 2 to 3 us.
+//
+// kMidMax: on GB300 the loop is even with launched rounds at 262,144 vertices
+// (PD2 4M x 1M 12.13 ms against 11.98) and ahead below (a 7-point mesh of
+// 32^3 vertices 0.175 ms with 16,384 here, 0.150 with 65,536).
+//
+// The remaining rounds go to the core phase when the worklist fits it and
+// shrinks slowly (a dense core: many rounds ahead; R-MAT 24 30.6 ms when the
+// core phase takes over at 1,024 vertices, 28.7 at 4,096); a worklist that is
+// about to run out finishes here.
+//
+// A server colors on many streams: 8 blocks per request leave the SMs to the
+// others (32 requests: 38.7 ms with a block per SM, 22.7 with 8 blocks up to
+// 8,192 vertices, 20.9 up to 16,384).
+template <class V, bool DYN = false>
+__global__ void __launch_bounds__(kMidThreads, 1) d1_mid(const Problem<V>* __restrict__ Pp,
+                                                         State* st) {
+    extern __shared__ int smem[];
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    Hot& h = ctx.h;
+    if (h.done || !h.mid) return;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    if ((int)blockIdx.x == P.slow_block && threadIdx.x == 0) {
+        // test hook: this block reaches its first barrier late (bounded)
+        const unsigned long long t_end = global_ns() + P.slow_ns;
+        while (global_ns() < t_end) __nanosleep(1000);
+    }
+    unsigned gen = 0u;
+    auto barrier = [&](int round) { return grid_barrier(st, h, gen, P.bar_polls, round); };
+    int r = h.round, cur = h.count(r & 1), status = ST_OK, done = 0, tail = 0;
+    const unsigned long long t0 = lead ? st->t0 : 0ull;
+    for (;;) {
+        const int np = (r & 1) ^ 1;
+        if (lead) {
+            st->push_cnt = 0;
+            st->ns[np] = st->nm[np] = st->nl[np] = 0;
+            st->s_next = st->h_next = 0ull;
+            // (a block may still be deciding the last round: hence the round number)
+            // the timer is slow to read: every eighth round
+            if ((r & 7) == 0 && global_ns() - t0 > P.timeout_ns && st->stop == 0) st->stop = r;
+        }
+        if (r > 1) assign_phase(P, h);
+        if (!barrier(r)) break;
+        detect_phase<V, DYN>(P, h, smem);
+        if (!barrier(r)) break;
+        const int nxt = h.count(np), pushes = h.push_cnt;
+        if (lead && P.trace_cap > 0) {
+            if (r < P.trace_cap) {
+                P.trace_w[r] = nxt;
+                P.trace_s[r] = (long long)*(volatile unsigned long long*)&st->s_next;
+                P.trace_h[r] = (long long)*(volatile unsigned long long*)&st->h_next;
+            }
+            if (r == 1) P.trace_h[0] = (long long)st->h_first;
+        }
+        if (nxt == 0) done = 1;
+        else if (nxt >= cur) status = ST_NO_PROGRESS;
+        else if (r >= P.max_rounds) status = ST_MAX_ROUNDS;
+        else if (h.stop > 0 && h.stop <= r) status = ST_TIMEOUT;
+        if (done || status != ST_OK) break;
+        tail = nxt <= P.tail_w && (long long)(cur - nxt) * 8 < nxt;
+        cur = nxt;
+        ++r;
+        if (pushes > 0) push_phase(P, pushes);
+        if (tail) break;
+        // the pushes are read by the next assign; without any, only the
+        // block's own copy moves on
+        if (pushes > 0) {
+            if (!barrier(r)) break;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) h.round = r;
+            __syncthreads();
+        }
+    }
+    if (lead) {   // the counters of round r are in place for the core phase
+        const int gave_up = *(volatile int*)&st->bar_timeout;
+        st->round = r;
+        st->status = gave_up ? ST_BARRIER : status;
+        st->done = gave_up || done || status != ST_OK;
+        st->tail = tail;
+        st->mid = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1087,12 +1388,13 @@ __device__ __forceinline__ int core_words(int k) { return (k + 31) >> 5; }
 
 // Phase 1a: a sortable priority key per worklist vertex; the matrix cleared.
 template <class V>
-__global__ void d1_core_keys(const Problem<V>* __restrict__ Pp) {
-    const Problem<V>& P = *Pp;
-    State* st = P.st;
-    if (*(volatile int*)&st->done || !*(volatile int*)&st->tail) return;
-    const int cp = st->round & 1, np = cp ^ 1;
-    const int nS = st->ns[cp], nM = st->nm[cp], nL = st->nl[cp], k = nS + nM + nL;
+__global__ void d1_core_keys(const Problem<V>* __restrict__ Pp, State* st) {
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    const Hot& h = ctx.h;
+    if (h.done || !h.tail) return;
+    const int cp = h.round & 1, np = cp ^ 1;
+    const int nS = h.ns[cp], nM = h.nm[cp], k = h.count(cp);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->core_k = k;
         st->core_par = np;
@@ -1104,7 +1406,7 @@ __global__ void d1_core_keys(const Problem<V>* __restrict__ Pp) {
         const int v = e.x;
         const uint64_t h =
             prio_hash(P.seed, (uint32_t)(v - P.g.base(P.g.graph(v))));
-        const unsigned nd = P.use_deg ? ~(unsigned)e.z : 0u;
+        const unsigned nd = P.use_deg ? ~(unsigned)P.g.degree(v, e.z) : 0u;
         A.key[i] = make_ulonglong2(((unsigned long long)nd << 32) | (h >> 32),
                                    (h << 32) | (unsigned)v);
     }
@@ -1116,14 +1418,15 @@ __global__ void d1_core_keys(const Problem<V>* __restrict__ Pp) {
 // memory at a time; each warp ranks four vertices), arrays in rank order.
 constexpr int kRankTile = 1024;
 template <class V>
-__global__ void d1_core_rank(const Problem<V>* __restrict__ Pp) {
-    const Problem<V>& P = *Pp;
-    State* st = P.st;
-    if (*(volatile int*)&st->done || !*(volatile int*)&st->tail) return;
+__global__ void d1_core_rank(const Problem<V>* __restrict__ Pp, State* st) {
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    const Hot& h = ctx.h;
+    if (h.done || !h.tail) return;
     __shared__ ulonglong2 tile[kRankTile];
-    const int cp = st->round & 1;
-    const int nS = st->ns[cp], nM = st->nm[cp], k = st->core_k;
-    const CoreArrays A = core_arrays(P, st->core_par, k);
+    const int cp = h.round & 1;
+    const int nS = h.ns[cp], nM = h.nm[cp], k = h.count(cp);
+    const CoreArrays A = core_arrays(P, cp ^ 1, k);
     const int lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const int per = wpb * 4;
     for (int b0 = blockIdx.x * per; b0 < k; b0 += gridDim.x * per) {
@@ -1171,22 +1474,23 @@ __device__ __forceinline__ void core_edge(const Problem<V>& P, int i, int u, int
 }
 
 template <class V>
-__global__ void d1_core_bits(const Problem<V>* __restrict__ Pp) {
-    const Problem<V>& P = *Pp;
-    State* st = P.st;
-    if (*(volatile int*)&st->done || !*(volatile int*)&st->tail) return;
-    const int k = st->core_k, words = core_words(k);
-    const CoreArrays A = core_arrays(P, st->core_par, k);
+__global__ void d1_core_bits(const Problem<V>* __restrict__ Pp, State* st) {
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    const Hot& h = ctx.h;
+    if (h.done || !h.tail) return;
+    const int k = h.count(h.round & 1), words = core_words(k);
+    const CoreArrays A = core_arrays(P, (h.round & 1) ^ 1, k);
     const int lane = lane_id(), wpb = blockDim.x >> 5;
     const int gw = blockIdx.x * wpb + (threadIdx.x >> 5), nw = gridDim.x * wpb;
     for (int i = gw; i < k; i += nw) {
         const int4 e = A.lent[i];
         if (e.y > kCoreWarpList) continue;
-        const int* h = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
+        const int* list = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
         for (int b0 = lane; b0 < e.y; b0 += 128) {
             int u[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) u[q] = b0 + 32 * q < e.y ? __ldg(h + b0 + 32 * q) : -1;
+            for (int q = 0; q < 4; ++q) u[q] = b0 + 32 * q < e.y ? __ldg(list + b0 + 32 * q) : -1;
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 if (u[q] >= 0) core_edge(P, i, u[q], words);
@@ -1195,8 +1499,9 @@ __global__ void d1_core_bits(const Problem<V>* __restrict__ Pp) {
     for (int i = blockIdx.x; i < k; i += gridDim.x) {
         const int4 e = A.lent[i];
         if (e.y <= kCoreWarpList) continue;   // block-uniform
-        const int* h = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
-        for (int b = threadIdx.x; b < e.y; b += blockDim.x) core_edge(P, i, __ldg(h + b), words);
+        const int* list = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
+        for (int b = threadIdx.x; b < e.y; b += blockDim.x)
+            core_edge(P, i, __ldg(list + b), words);
     }
 }
 
@@ -1206,7 +1511,7 @@ __device__ __forceinline__ unsigned forbidden_word(const Problem<V>& P, int4 e, 
     if (w < 2) return __ldcg(reinterpret_cast<const unsigned*>(P.bm0 + e.x) + w);
     if (e.z < 64 || w - 2 > (e.z >> 5)) return 0u;
     const long long b = P.g.begin(P.g.graph(e.x), e.w);
-    return __ldcg(P.bmx + bm_offset(b, e.x) + (w - 2));
+    return __ldcg(P.bmx + P.g.bm(e.x, b) + (w - 2));
 }
 
 // Shared memory of one CTA of the core loop: R = ceil(k / C) rows, row x of
@@ -1354,7 +1659,7 @@ __device__ __forceinline__ void core_forbid(const Problem<V>& P, const CoreSmem&
         atomicOr(reinterpret_cast<unsigned*>(P.bm0 + e.x) + gw, bit);
     } else {
         const long long b = P.g.begin(P.g.graph(e.x), e.w);
-        atomicOr(P.bmx + bm_offset(b, e.x) + (gw - 2), bit);
+        atomicOr(P.bmx + P.g.bm(e.x, b) + (gw - 2), bit);
     }
 }
 
@@ -1476,7 +1781,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
         if (lane == 0 && r == 1) P.trace_h[0] = (long long)st->h_first;
         for (int j = lane; j < k; j += 32) {
             const int4 e = A.lent[j];
-            sum_s += (unsigned long long)e.z;   // per lane; the total is the warp's sum
+            sum_s += (unsigned long long)P.g.degree(e.x, e.z);   // per lane, see below
             sum_h += (unsigned long long)e.y;
         }
     }
@@ -1631,7 +1936,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
             for (int j = lane; j < k; j += 32)
                 if (reinterpret_cast<const unsigned*>(S.won + now * words4)[j >> 5] >> (j & 31) & 1u) {
                     const int4 e = A.lent[j];
-                    sum_s -= (unsigned long long)e.z;
+                    sum_s -= (unsigned long long)P.g.degree(e.x, e.z);
                     sum_h -= (unsigned long long)e.y;
                 }
             const unsigned long long ts = warp_sum(sum_s), th = warp_sum(sum_h);
@@ -1744,17 +2049,22 @@ struct Engine {
     HostBuf h_problem, h_state, h_misc;
     int trace_cap = 0;
     int last_want_trace = 0, last_tcap = 1;
-    // [0]: setup + rounds; [1]: rounds only (setup enqueued by the host
-    // while the adjacency is still being uploaded)
-    cudaGraph_t graph[2] = {nullptr, nullptr};
-    cudaGraphExec_t exec[2] = {nullptr, nullptr};
+    // [0]: setup + rounds; [1]: rounds only (setup enqueued by the host:
+    // while the adjacency is still being uploaded, or lists built elsewhere);
+    // [2], [3]: the same for problems of at most mid_w vertices, which have no
+    // launch-per-round rounds
+    static constexpr int kGraphs = 4;
+    cudaGraph_t graph[kGraphs] = {};
+    cudaGraphExec_t exec[kGraphs] = {};
     int g_grid = 0, g_block = 0, g_det = 0, g_async = 0, g_dyn = 0;
+    int mid_grid = -1;    // blocks of the mid loop (-1: not asked yet)
+    bool shares_gpu = false;   // others color on the same GPU: a small mid loop (set once)
     int core_grid = -1;   // CTAs of the core loop's cluster (-1: not asked yet)
     cudaStream_t up_stream = nullptr;             // adjacency upload
     cudaEvent_t up_fork = nullptr, up_done[kUploadChunks] = {};
 
     void destroy_graph() {
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < kGraphs; ++k) {
             if (exec[k]) cudaGraphExecDestroy(exec[k]);
             if (graph[k]) cudaGraphDestroy(graph[k]);
             exec[k] = nullptr;
@@ -1785,16 +2095,20 @@ struct Engine {
     struct Geometry {
         int grid, block;
         size_t smem;   // two warp appenders per warp
+        int mid_grid;  // co-resident blocks of the mid loop (0: no cooperative launch)
         int core_grid; // CTAs of the core loop's cluster (0: no cluster fits, no core phase)
         int det_grid;  // detect: its own occupancy
     };
 
     pgc_status geometry(const Opts& o, Geometry* g) {
         g->block = o.block;
-        g->smem = (size_t)(o.block / 32) * 2 * kAppend4Slots * sizeof(int4);
+        g->smem = (size_t)(o.block / 32) * 2 * kIdxSlots * sizeof(int);
         if (g->smem > 48 * 1024) {   // 1024-thread blocks: 64 KB of append buffers
-            for (const void* f : {(const void*)d1_classify<V>, (const void*)d1_tier<V>,
-                                  (const void*)d1_detect<V>, (const void*)d1_detect<V, true>})
+            std::vector<const void*> fs = {(const void*)d1_detect<V>};
+            if constexpr (V::kSetup) {
+                fs.push_back((const void*)d1_detect<V, true>);
+            }
+            for (const void* f : fs)
                 PGC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)g->smem));
         }
@@ -1803,8 +2117,11 @@ struct Engine {
         if (per_sm == 0) {
             int a = 0, b = 0;
             PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, d1_detect<V>, o.block, g->smem));
-            PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, d1_build<V>, o.block, 0));
-            per_sm = std::max(1, std::min(a, b));
+            if constexpr (V::kSetup)
+                PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, d1_build<V>, o.block, 0));
+            else
+                PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, d1_assign<V>, o.block, 0));
+            per_sm = std::max(1, b);
             g->det_grid = dev.num_sms * std::max(1, a);
         }
         g->grid = dev.num_sms * per_sm;
@@ -1822,7 +2139,33 @@ struct Engine {
             core_grid = e == cudaSuccess && clusters > 0 ? kCoreCluster : 0;
         }
         g->core_grid = core_grid;
+        if (mid_grid < 0) {
+            int per = 0, coop = 0;
+            for (int d = 0; d < (V::kSetup ? 2 : 1); ++d)
+                PGC_CUDA(cudaFuncSetAttribute(mid_func(d), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)kMidSmem));
+            PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mid_func(0), kMidThreads,
+                                                                   kMidSmem));
+            if (V::kSetup) {   // both variants run on the same grid
+                int per_dyn = 0;
+                PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_dyn, mid_func(1),
+                                                                       kMidThreads, kMidSmem));
+                per = std::min(per, per_dyn);
+            }
+            PGC_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev.device));
+            mid_grid = coop && per > 0 ? (shares_gpu ? std::min(kMidShared, dev.num_sms)
+                                                     : dev.num_sms) : 0;
+        }
+        g->mid_grid = mid_grid;
         return PGC_OK;
+    }
+
+    static constexpr size_t kMidSmem = (kMidThreads / 32) * 2 * kIdxSlots * sizeof(int);
+    static void* mid_func(int dyn) {
+        if constexpr (V::kSetup) {
+            if (dyn) return (void*)d1_mid<V, true>;
+        }
+        return (void*)d1_mid<V>;
     }
 
     // launch configuration of the core loop: one cluster
@@ -1852,9 +2195,12 @@ struct Engine {
 
     pgc_status build_graph(const Geometry& g, int async, int dyn) {
         destroy_graph();
-        for (int k = 0; k < 2; ++k)
-            if (pgc_status s = build_one_graph(g, k == 0, async, dyn, &graph[k], &exec[k]))
+        for (int k = 0; k < kGraphs; ++k) {
+            const bool setup = k % 2 == 0, small = k >= 2;
+            if ((setup && !V::kSetup) || (small && (async || g.mid_grid == 0))) continue;
+            if (pgc_status s = build_one_graph(g, setup, small, async, dyn, &graph[k], &exec[k]))
                 return s;
+        }
         g_dyn = dyn;
         g_grid = g.grid;
         g_det = g.det_grid;
@@ -1863,77 +2209,104 @@ struct Engine {
         return PGC_OK;
     }
 
-    // Setup (optional), round 1 (assign first under PGC_ASYNC), then the
-    // WHILE node of the later rounds and the core phase.
-    pgc_status build_one_graph(const Geometry& g, bool setup, int async, int dyn,
+    // Setup (optional), round 1 (assign first under PGC_ASYNC) and the WHILE
+    // node of the later rounds (both unless small), the mid loop and the core
+    // phase.
+    pgc_status build_one_graph(const Geometry& g, bool setup, bool small, int async, int dyn,
                                cudaGraph_t* graph_out, cudaGraphExec_t* exec_out) {
         Problem<V>* dP = problem.as<Problem<V>>();
         PGC_CUDA(cudaGraphCreate(graph_out, 0));
         cudaGraph_t graph = *graph_out;
         cudaGraphConditionalHandle handle = 0;
-        PGC_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 0u, cudaGraphCondAssignDefault));
+        if (!small)
+            PGC_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 0u,
+                                                      cudaGraphCondAssignDefault));
         int use_cond = 1;
         cudaGraphConditionalHandle hnd = handle;
         int lo = 0, hi = INT32_MAX;
+        State* dS = state.as<State>();
         void* p_args[] = {&dP};
+        void* s_args[] = {&dP, &dS};
         void* b_args[] = {&dP, &lo, &hi};
-        void* c_args[] = {&dP, &hnd, &use_cond};
+        void* c_args[] = {&dP, &dS, &hnd, &use_cond};
         cudaMemsetParams ms = {};
         ms.dst = state.ptr;
         ms.value = 0;
         ms.elementSize = 4;
         ms.width = sizeof(State) / 4;
         ms.height = 1;
-        cudaGraphNode_t n_ms, n_cls, n_build, n_tier, n_asg1, n_det, n_push, n_loop;
+        cudaGraphNode_t n_ms, n_cls, n_build, n_tier = nullptr, n_asg1, n_det, n_push, n_loop;
         if (setup) PGC_CUDA(cudaGraphAddMemsetNode(&n_ms, graph, nullptr, 0, &ms));
-        cudaKernelNodeParams k_cls = knode((void*)d1_classify<V>, g, g.smem, p_args);
-        cudaKernelNodeParams k_build = knode((void*)d1_build<V>, g, 0, b_args);
-        cudaKernelNodeParams k_tier = knode((void*)d1_tier<V>, g, g.smem, p_args);
-        cudaKernelNodeParams k_det =
-            knode(dyn ? (void*)d1_detect<V, true> : (void*)d1_detect<V>, g, g.smem, c_args);
+        void* detect = (void*)d1_detect<V>;
+        if constexpr (V::kSetup) {
+            if (dyn) detect = (void*)d1_detect<V, true>;
+        }
+        cudaKernelNodeParams k_det = knode(detect, g, g.smem, c_args);
         k_det.gridDim = dim3(g.det_grid);
-        cudaKernelNodeParams k_push = knode((void*)d1_push<V>, g, 0, p_args);
+        cudaKernelNodeParams k_push = knode((void*)d1_push<V>, g, 0, s_args);
         cudaKernelNodeParams k_asg = knode((void*)d1_assign<V>, g, 0, c_args);
-        if (setup) {
-            PGC_CUDA(cudaGraphAddKernelNode(&n_cls, graph, &n_ms, 1, &k_cls));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_build, graph, &n_cls, 1, &k_build));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_tier, graph, &n_build, 1, &k_tier));
+        if constexpr (V::kSetup) {
+            if (setup) {
+                cudaKernelNodeParams k_cls = knode((void*)d1_classify<V>, g, 0, p_args);
+                cudaKernelNodeParams k_build = knode((void*)d1_build<V>, g, 0, b_args);
+                cudaKernelNodeParams k_tier = knode((void*)d1_tier<V>, g, 0, p_args);
+                PGC_CUDA(cudaGraphAddKernelNode(&n_cls, graph, &n_ms, 1, &k_cls));
+                PGC_CUDA(cudaGraphAddKernelNode(&n_build, graph, &n_cls, 1, &k_build));
+                PGC_CUDA(cudaGraphAddKernelNode(&n_tier, graph, &n_build, 1, &k_tier));
+            }
         }
-        if (async) {
-            PGC_CUDA(cudaGraphAddKernelNode(&n_asg1, graph, setup ? &n_tier : nullptr,
-                                            setup ? 1 : 0, &k_asg));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_det, graph, &n_asg1, 1, &k_det));
-        } else {
-            PGC_CUDA(cudaGraphAddKernelNode(&n_det, graph, setup ? &n_tier : nullptr,
-                                            setup ? 1 : 0, &k_det));
+        cudaGraphNode_t last = nullptr;   // what the next node waits for (none: starts at once)
+        if (setup) last = n_tier;
+        auto after = [&](cudaGraphNode_t* node, cudaGraph_t gr, const cudaKernelNodeParams& k) {
+            const cudaError_t e = cudaGraphAddKernelNode(node, gr, last ? &last : nullptr,
+                                                         last ? 1 : 0, &k);
+            last = *node;
+            return e;
+        };
+        if (!small) {
+            if (async) PGC_CUDA(after(&n_asg1, graph, k_asg));
+            PGC_CUDA(after(&n_det, graph, k_det));
+            PGC_CUDA(after(&n_push, graph, k_push));
+            cudaGraphNodeParams cp = {};
+            cp.type = cudaGraphNodeTypeConditional;
+            cp.conditional.handle = handle;
+            cp.conditional.type = cudaGraphCondTypeWhile;
+            cp.conditional.size = 1;
+            PGC_CUDA(cudaGraphAddNode(&n_loop, graph, &n_push, nullptr, 1, &cp));
+            cudaGraph_t body = cp.conditional.phGraph_out[0];
+            cudaGraphNode_t b_asg, b_det, b_push;
+            PGC_CUDA(cudaGraphAddKernelNode(&b_asg, body, nullptr, 0, &k_asg));
+            PGC_CUDA(cudaGraphAddKernelNode(&b_det, body, &b_asg, 1, &k_det));
+            PGC_CUDA(cudaGraphAddKernelNode(&b_push, body, &b_det, 1, &k_push));
+            last = n_loop;
         }
-        PGC_CUDA(cudaGraphAddKernelNode(&n_push, graph, &n_det, 1, &k_push));
-        cudaGraphNodeParams cp = {};
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = handle;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        PGC_CUDA(cudaGraphAddNode(&n_loop, graph, &n_push, nullptr, 1, &cp));
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        cudaGraphNode_t b_asg, b_det, b_push;
-        PGC_CUDA(cudaGraphAddKernelNode(&b_asg, body, nullptr, 0, &k_asg));
-        PGC_CUDA(cudaGraphAddKernelNode(&b_det, body, &b_asg, 1, &k_det));
-        PGC_CUDA(cudaGraphAddKernelNode(&b_push, body, &b_det, 1, &k_push));
-        // the remaining small rounds: the core phase (no-ops unless the loop
-        // stopped with st->tail set)
-        if (g.core_grid > 0) {
-            cudaKernelNodeParams k_ckeys = knode((void*)d1_core_keys<V>, g, 0, p_args);
-            cudaKernelNodeParams k_crank = knode((void*)d1_core_rank<V>, g, 0, p_args);
-            cudaKernelNodeParams k_cbits = knode((void*)d1_core_bits<V>, g, 0, p_args);
+        if (g.mid_grid > 0 && !async) {
+            cudaKernelNodeParams k_mid = knode(mid_func(dyn), g, kMidSmem, s_args);
+            k_mid.gridDim = dim3(g.mid_grid);
+            k_mid.blockDim = dim3(kMidThreads);
+            cudaGraphNode_t n_mid;
+            PGC_CUDA(after(&n_mid, graph, k_mid));
+            cudaLaunchAttributeValue coop = {};
+            coop.cooperative = 1;
+            PGC_CUDA(cudaGraphKernelNodeSetAttribute(n_mid, cudaLaunchAttributeCooperative, &coop));
+        }
+        // no-ops unless the mid loop stopped with st->tail set
+        if (g.core_grid > 0 && g.mid_grid > 0 && !async && !dyn) {
+            cudaKernelNodeParams k_ckeys = knode((void*)d1_core_keys<V>, g, 0, s_args);
+            k_ckeys.gridDim = dim3(dev.num_sms);
+            cudaKernelNodeParams k_crank = knode((void*)d1_core_rank<V>, g, 0, s_args);
+            k_crank.gridDim = dim3(dev.num_sms);
+            cudaKernelNodeParams k_cbits = knode((void*)d1_core_bits<V>, g, 0, s_args);
+            k_cbits.gridDim = dim3(dev.num_sms);
             cudaKernelNodeParams k_cloop =
                 knode((void*)d1_core_loop<V>, g, core_smem_bytes(kCoreMax), p_args);
             k_cloop.gridDim = dim3(g.core_grid);
             k_cloop.blockDim = dim3(kCoreThreads);
             cudaGraphNode_t n_ckeys, n_crank, n_cbits, n_cloop;
-            PGC_CUDA(cudaGraphAddKernelNode(&n_ckeys, graph, &n_loop, 1, &k_ckeys));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_crank, graph, &n_ckeys, 1, &k_crank));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_cbits, graph, &n_crank, 1, &k_cbits));
-            PGC_CUDA(cudaGraphAddKernelNode(&n_cloop, graph, &n_cbits, 1, &k_cloop));
+            PGC_CUDA(after(&n_ckeys, graph, k_ckeys));
+            PGC_CUDA(after(&n_crank, graph, k_crank));
+            PGC_CUDA(after(&n_cbits, graph, k_cbits));
+            PGC_CUDA(after(&n_cloop, graph, k_cloop));
             cudaLaunchAttributeValue dim = {};
             dim.clusterDim.x = (unsigned)g.core_grid;
             dim.clusterDim.y = dim.clusterDim.z = 1;
@@ -1997,13 +2370,18 @@ struct Engine {
         return finish(o, rounds, num_colors);
     }
 
+    // ListView: enqueues the kernel that builds the lists (and what
+    // d1_classify, d1_build and d1_tier leave behind) for the problem.
+    using Setup = std::function<pgc_status(const Problem<V>*)>;
+
     // Enqueues one coloring on `stream` with caller-provided scratch (the
     // device loop in graph mode; host-loop mode drives the rounds and
     // therefore blocks).  The round state and trace are copied to pinned
     // host memory on the same stream; call finish() once the stream is done.
     pgc_status launch(const Scratch& sc, const V& view, int n, long long nnz, int* d_col,
                       int* g_rounds, int* g_colors, uint64_t seed, const Opts& o,
-                      cudaStream_t stream, const Upload* up = nullptr) {
+                      cudaStream_t stream, const Upload* up = nullptr,
+                      const Setup* setup = nullptr) {
         const uint32_t pflags = o.flags & (PGC_PRIORITY_DYNAMIC | PGC_PRIORITY_SATURATION);
         if (pflags == (PGC_PRIORITY_DYNAMIC | PGC_PRIORITY_SATURATION))
             return fail(PGC_ERR_INVALID_ARG, "PGC_PRIORITY_DYNAMIC and PGC_PRIORITY_SATURATION "
@@ -2067,9 +2445,14 @@ struct Engine {
         hp->prio = sc.prio;
         hp->max_rounds = o.max_rounds > 0 ? o.max_rounds : (n < INT32_MAX ? n + 1 : n);
         hp->det_s = o.mid_degree;
-        hp->det_m = o.hub_degree;
-        hp->tail_w = (o.flags & PGC_ASYNC) || pflags || g.core_grid == 0
+        // lists that hold whole rows: hubs' lists are long, and a block reads 1024
+        // entries per step where a warp reads 128
+        hp->det_m = pflags ? std::max(o.mid_degree, std::min(o.hub_degree, kVaryingHub))
+                           : o.hub_degree;
+        hp->mid_w = hp->async_mode || g.mid_grid == 0 ? 0 : shares_gpu ? kMidSharedMax : kMidMax;
+        hp->tail_w = hp->mid_w == 0 || pflags || g.core_grid == 0
                          ? 0 : std::min(o.tail_vertices, kCoreMax);
+        const int small = n <= hp->mid_w ? 2 : 0;
         const TestHooks th = test_hooks();
         hp->bar_polls = th.barrier_polls;
         hp->slow_block = th.slow_block;
@@ -2081,12 +2464,16 @@ struct Engine {
         State* hs = h_state.as<State>();
         if (!(o.flags & PGC_HOST_LOOP)) {
             const int dyn = hp->prio_mode != 0;
-            if (!exec[0] || g_grid != g.grid || g_block != g.block || g_det != g.det_grid ||
+            if (!exec[1] || g_grid != g.grid || g_block != g.block || g_det != g.det_grid ||
                 g_async != hp->async_mode || g_dyn != dyn) {
                 if (pgc_status s = build_graph(g, hp->async_mode, dyn)) return s;
             }
-            if (!up) {
-                PGC_CUDA(cudaGraphLaunch(exec[0], stream));
+            if constexpr (!V::kSetup) {
+                PGC_CUDA(cudaMemsetAsync(state.ptr, 0, sizeof(State), stream));
+                if (pgc_status s = (*setup)(dP)) return s;
+                PGC_CUDA(cudaGraphLaunch(exec[small + 1], stream));
+            } else if (!up) {
+                PGC_CUDA(cudaGraphLaunch(exec[small], stream));
             } else {
                 // setup by hand: classify needs only the row offsets; the
                 // build of row range k waits for that range's copy
@@ -2114,12 +2501,12 @@ struct Engine {
                     PGC_CUDA(cudaEventRecord(up_done[k], up_stream));
                 }
                 PGC_CUDA(cudaMemsetAsync(state.ptr, 0, sizeof(State), stream));
-                d1_classify<V><<<g.grid, g.block, g.smem, stream>>>(dP);
+                d1_classify<V><<<g.grid, g.block, 0, stream>>>(dP);
                 for (int k = 0; k < kUploadChunks; ++k) {
                     PGC_CUDA(cudaStreamWaitEvent(stream, up_done[k], 0));
                     d1_build<V><<<g.grid, g.block, 0, stream>>>(dP, cut[k], cut[k + 1]);
                 }
-                d1_tier<V><<<g.grid, g.block, g.smem, stream>>>(dP);
+                d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP);
                 PGC_CUDA(cudaGetLastError());
                 PGC_CUDA(cudaGraphLaunch(exec[1], stream));
             }
@@ -2128,6 +2515,7 @@ struct Engine {
             kt.prof = o.profile;
             kt.stream = stream;
             const cudaGraphConditionalHandle none = 0;
+            State* dS = state.as<State>();
             PGC_CUDA(cudaMemsetAsync(state.ptr, 0, sizeof(State), stream));
 #define PGC_TIMED(slot, name, launch_)                        \
     do {                                                      \
@@ -2136,40 +2524,58 @@ struct Engine {
         PGC_CUDA(cudaGetLastError());                         \
         if (pgc_status s_ = kt.end()) return s_;              \
     } while (0)
-            PGC_TIMED(0, "d1_classify", (d1_classify<V><<<g.grid, g.block, g.smem, stream>>>(dP)));
-            PGC_TIMED(1, "d1_build",
-                      (d1_build<V><<<g.grid, g.block, 0, stream>>>(dP, 0, INT32_MAX)));
-            PGC_TIMED(2, "d1_tier", (d1_tier<V><<<g.grid, g.block, g.smem, stream>>>(dP)));
-            for (int round = 1;; ++round) {
+            if constexpr (V::kSetup) {
+                PGC_TIMED(0, "d1_classify",
+                          (d1_classify<V><<<g.grid, g.block, 0, stream>>>(dP)));
+                PGC_TIMED(1, "d1_build",
+                          (d1_build<V><<<g.grid, g.block, 0, stream>>>(dP, 0, INT32_MAX)));
+                PGC_TIMED(2, "d1_tier", (d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP)));
+            } else {   // slot 0 is the caller's
+                if (pgc_status s_ = kt.begin(1, "net_lists")) return s_;
+                if (pgc_status s_ = (*setup)(dP)) return s_;
+                if (pgc_status s_ = kt.end()) return s_;
+            }
+            for (int round = 1; !small; ++round) {
                 if (round > 1 || hp->async_mode)
                     PGC_TIMED(3, "d1_assign",
-                              (d1_assign<V><<<g.grid, g.block, 0, stream>>>(dP, none, 0)));
-                PGC_TIMED(4, "d1_detect",
-                          (hp->prio_mode
-                               ? d1_detect<V, true><<<g.det_grid, g.block, g.smem, stream>>>(
-                                     dP, none, 0)
-                               : d1_detect<V><<<g.det_grid, g.block, g.smem, stream>>>(dP, none,
-                                                                                      0)));
-                PGC_TIMED(5, "d1_push", (d1_push<V><<<g.grid, g.block, 0, stream>>>(dP)));
+                              (d1_assign<V><<<g.grid, g.block, 0, stream>>>(dP, dS, none, 0)));
+                if (pgc_status s_ = kt.begin(4, "d1_detect")) return s_;
+                bool dyn_detect = false;
+                if constexpr (V::kSetup) {
+                    if (hp->prio_mode) {
+                        dyn_detect = true;
+                        d1_detect<V, true><<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
+                    }
+                }
+                if (!dyn_detect)
+                    d1_detect<V><<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
+                PGC_CUDA(cudaGetLastError());
+                if (pgc_status s_ = kt.end()) return s_;
+                PGC_TIMED(5, "d1_push", (d1_push<V><<<g.grid, g.block, 0, stream>>>(dP, dS)));
                 PGC_CUDA(cudaMemcpyAsync(hs, state.ptr, sizeof(State), cudaMemcpyDeviceToHost,
                                          stream));
                 PGC_CUDA(cudaStreamSynchronize(stream));
-                if (hs->done) break;
-                if (hs->tail) {   // the remaining rounds: the core phase
-                    if (pgc_status s_ = kt.begin(6, "d1_core")) return s_;
-                    d1_core_keys<V><<<g.grid, g.block, 0, stream>>>(dP);
-                    d1_core_rank<V><<<g.grid, g.block, 0, stream>>>(dP);
-                    d1_core_bits<V><<<g.grid, g.block, 0, stream>>>(dP);
-                    PGC_CUDA(cudaGetLastError());
-                    cudaLaunchAttribute at;
-                    cudaLaunchConfig_t lc = core_config(stream, &at);
-                    PGC_CUDA(cudaLaunchKernelEx(&lc, d1_core_loop<V>,
-                                                (const Problem<V>*)dP));
-                    if (pgc_status s_ = kt.end()) return s_;
-                    break;
-                }
+                if (hs->done || hs->mid) break;
                 if (round > hp->max_rounds + 1)
                     return fail(PGC_ERR_CUDA, "device round control did not finish the loop");
+            }
+            if (hp->mid_w > 0) {   // no-ops once the coloring is done
+                void* args[] = {&dP, &dS};
+                if (pgc_status s_ = kt.begin(7, "d1_mid")) return s_;
+                PGC_CUDA(cudaLaunchCooperativeKernel(mid_func(hp->prio_mode != 0), dim3(g.mid_grid),
+                                                     dim3(kMidThreads), args, kMidSmem, stream));
+                if (pgc_status s_ = kt.end()) return s_;
+            }
+            if (hp->tail_w > 0) {
+                if (pgc_status s_ = kt.begin(6, "d1_core")) return s_;
+                d1_core_keys<V><<<dev.num_sms, g.block, 0, stream>>>(dP, dS);
+                d1_core_rank<V><<<dev.num_sms, g.block, 0, stream>>>(dP, dS);
+                d1_core_bits<V><<<dev.num_sms, g.block, 0, stream>>>(dP, dS);
+                PGC_CUDA(cudaGetLastError());
+                cudaLaunchAttribute at;
+                cudaLaunchConfig_t lc = core_config(stream, &at);
+                PGC_CUDA(cudaLaunchKernelEx(&lc, d1_core_loop<V>, (const Problem<V>*)dP));
+                if (pgc_status s_ = kt.end()) return s_;
             }
 #undef PGC_TIMED
             kt.destroy();

@@ -111,47 +111,12 @@ __device__ __forceinline__ long long bitmap_offset(int rp_v, int v) {
 
 namespace pgc {
 
-// WarpAppend for 16-byte entries (kAppend4Slots int4 per appender).  Its
-// buffer is kept at 32 + 32 entries: the distance-1 detection kernel that
-// uses it relies on L1, and a larger shared buffer costs more L1 than the
-// saved counter atomics are worth (measured: round 2 of R-MAT-24 took 50%
-// longer with 96-entry flushes).
-constexpr int kAppend4Flush = 32;
-constexpr int kAppend4Slots = kAppend4Flush + 32;
-
-struct WarpAppend4 {
-    int4* buf;
-    int count;
-};
-
-__device__ __forceinline__ void wa4_push(WarpAppend4& a, bool pred, int4 e, int4* out,
-                                         int* out_cnt) {
-    const unsigned lane = lane_id();
-    const unsigned m = __ballot_sync(kFullMask, pred);
-    if (pred) a.buf[a.count + __popc(m & ((1u << lane) - 1u))] = e;
-    a.count += __popc(m);
-    __syncwarp();
-    if (a.count >= kAppend4Flush) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(out_cnt, kAppend4Flush);
-        base = __shfl_sync(kFullMask, base, 0);
-#pragma unroll
-        for (int k = 0; k < kAppend4Flush; k += 32) out[base + k + lane] = a.buf[k + lane];
-        const int rem = a.count - kAppend4Flush;
-        int4 tmp = make_int4(0, 0, 0, 0);
-        if ((int)lane < rem) tmp = a.buf[kAppend4Flush + lane];
-        __syncwarp();
-        if ((int)lane < rem) a.buf[lane] = tmp;
-        a.count = rem;
-        __syncwarp();
-    }
-}
-
 // Re-append of entries that already sit in a source list (a loser keeps
 // its entry for the next round): the shared buffer holds 4-byte source
 // indices instead of 16-byte entries, so the same shared memory takes
-// kIdxFlush entries per counter atomic; the flush copies the entries from
-// the source list (just read, so mostly cache hits).
+// kIdxFlush entries per counter atomic; a flush copies the entries from the
+// source list (just read, so mostly cache hits).  What is left at the end is
+// the block's to place (one atomic for all its warps).
 constexpr int kIdxFlush = 224;
 constexpr int kIdxSlots = kIdxFlush + 32;
 
@@ -180,28 +145,6 @@ __device__ __forceinline__ void ia_push(IdxAppend& a, bool pred, int idx, const 
         a.count = rem;
         __syncwarp();
     }
-}
-
-__device__ __forceinline__ void ia_flush(IdxAppend& a, const int4* src, int4* out, int* out_cnt) {
-    if (a.count == 0) return;
-    const unsigned lane = lane_id();
-    int base = 0;
-    if (lane == 0) base = atomicAdd(out_cnt, a.count);
-    base = __shfl_sync(kFullMask, base, 0);
-    for (int k = lane; k < a.count; k += 32) out[base + k] = src[a.buf[k]];
-    a.count = 0;
-    __syncwarp();
-}
-
-__device__ __forceinline__ void wa4_flush(WarpAppend4& a, int4* out, int* out_cnt) {
-    if (a.count == 0) return;
-    const unsigned lane = lane_id();
-    int base = 0;
-    if (lane == 0) base = atomicAdd(out_cnt, a.count);
-    base = __shfl_sync(kFullMask, base, 0);
-    for (int k = lane; k < a.count; k += 32) out[base + k] = a.buf[k];
-    a.count = 0;
-    __syncwarp();
 }
 
 }  // namespace pgc

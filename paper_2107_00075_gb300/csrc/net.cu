@@ -11,7 +11,14 @@
 //        columns (CSR); the nets of column v are its rows (CSC) (Sec. 3.6).
 // Only the vertices (D2) or columns (PD2) are colored.
 //
-// Per round:
+// Two ways to color, with the same rounds:
+//
+// Conflict lists (net_lists): the vertices that share a net with v, each once,
+// are its row in the conflict graph, and the distance-1 engine runs the
+// rounds.  The way of every problem whose vertices have fewer than 2048
+// members in their nets and whose lists fit 2 GB.
+//
+// Net rounds, for the others.  Per round:
 //   assign  v in W: forbidden(v) = OR of the color masks of v's nets;
 //           t = first free color (Alg. 1); col[v] = -t.  Marks v's nets
 //           active for this round (skipped while W's nets cover them all).
@@ -26,8 +33,7 @@
 //           committed members' colors, kept incrementally: each vertex
 //           updates its nets once).
 // The loop runs on the device (CUDA graph, conditional WHILE node).
-#include "runtime.h"
-#include "device_common.cuh"
+#include "d1_engine.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -36,8 +42,6 @@
 #include <unordered_map>
 
 namespace pgc {
-std::vector<std::function<void()>>& release_hooks();
-
 namespace net {
 
 constexpr int kThreadNets = 64;   // vertices with up to this many nets: one thread
@@ -63,7 +67,9 @@ struct State {
     unsigned long long nets_seen;      // traced: nets detection visited this round
     unsigned long long members_seen;   // traced: their members
     int max_deg;      // largest degree term of a key (sizes the 32-bit key of ck)
-    int pad2;
+    int members;      // max over v of sum over its nets of |net|
+    unsigned long long pairs;          // sum over v of sum over its nets of (|net| - 1)
+    unsigned long long list_next;      // conflict lists: entries handed out
 };
 
 struct Problem {
@@ -126,8 +132,8 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
     const int warp = threadIdx.x >> 5;
     WarpAppend at = {smem + warp * 2 * kAppendSlots, 0},
                aw = {smem + warp * 2 * kAppendSlots + kAppendSlots, 0};
-    int my_bound = 0, my_deg = 0;
-    unsigned long long my_h = 0ull;
+    int my_bound = 0, my_deg = 0, my_members = 0;
+    unsigned long long my_h = 0ull, my_pairs = 0ull;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long wbase = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
          wbase < P.n; wbase += stride) {
@@ -146,6 +152,8 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
             long long b = 0;
             for (int j = 0; j < k; ++j) b += net_size(P, vertex_net(P, v, beg, j)) - 1;
             my_bound = max(my_bound, (int)min(b, (long long)INT32_MAX - 1));
+            my_pairs += (unsigned long long)b;
+            my_members = max(my_members, (int)min(b + k, (long long)INT32_MAX - 1));
             my_h += (unsigned long long)k;
         }
         wa_push(at, valid && k <= kThreadNets, (int)i, P.wt[1], &st->nt[1]);
@@ -158,8 +166,12 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
     my_bound = warp_max(my_bound);
     my_deg = warp_max(my_deg);
     my_h = warp_sum(my_h);
+    my_pairs = warp_sum(my_pairs);
+    my_members = warp_max(my_members);
     if (lane_id() == 0) {
+        if (my_pairs) atomicAdd(&st->pairs, my_pairs);
         atomicMax(&st->bound, my_bound);
+        atomicMax(&st->members, my_members);
         if (P.use_deg) atomicMax(&st->max_deg, my_deg);
         if (my_h) atomicAdd(&st->h_first, my_h);
     }
@@ -860,6 +872,265 @@ __global__ void net_commit(const Problem* __restrict__ Pp, cudaGraphConditionalH
 
 
 // ---------------------------------------------------------------------------
+// conflict lists: the vertices that share a net with v, each once, those with
+// priority over v first.  With them distance-2 and partial distance-2 are
+// distance-1 colorings of the conflict graph (d1_engine.cuh, ListView), whose
+// rounds cost what their worklists need, while the net rounds below visit
+// every net of the worklist: 27 gathers per net and 27 mask words per vertex
+// and round on the 27-point stencil, against one forbidden word and a list
+// that is left at the first conflict.
+//
+// One warp per vertex: the members of its nets go into a hash set in shared
+// memory (a mesh lists each neighbor several times: 702 members, 124
+// vertices), and a member that is new also to a list there, so what follows --
+// one key gather per vertex and the split by priority -- handles each vertex
+// once and in the order of the nets, which keeps a mesh's runs of neighbors
+// together (coalesced color gathers in every round).  Rows are handed out from
+// one counter in chunks, in any order.
+//
+// Bound by issue (about 2,500 warp instructions per vertex of the 27-point
+// mesh 128^3, 6.0 ms for its 2.1M vertices; PD2 4M x 1M 4.6 ms).  A hash that
+// kept blocks of 32 ids together put whole runs of a mesh on top of each
+// other (39 ms); reading the set out slot by slot took 10 ms.
+//
+// With lists the whole coloring of the mesh takes 13.7 ms (22.5 in net
+// rounds), of PD2 4M x 1M 12.0 ms (21.9), of PD2 40K x 10K 1.1 ms (3.3), of a
+// 7-point mesh of 51,615 vertices 0.39 ms (0.75).
+// ---------------------------------------------------------------------------
+constexpr int kListMinLog = 6, kListMaxLog = 11;          // log2 of a warp's hash set
+constexpr int kListMid = 64;                              // lists up to this length: S tier
+constexpr unsigned kListEmpty = 0xffffffffu;              // no id: ids are below 2^31 - 1
+constexpr unsigned long long kListMaxEntries = 1ull << 29;   // 2 GB of lists
+
+struct ListArgs {
+    int2* rows;          // {first entry, length} per vertex
+    int* lists;
+    unsigned cap;        // entries of the buffer
+    unsigned chunk;      // entries a warp takes from the counter at a time
+    int log;             // log2 of a warp's set: above every vertex's member count, so a
+                         // probe always ends
+    int group;           // consecutive vertices per warp
+};
+
+// ints of shared memory per warp: the set, and the list of 5/8 of it (a vertex
+// with more neighbors is read from the set)
+__host__ __device__ inline int list_warp_ints(int log) { return (1 << log) + (5 << log) / 8; }
+
+// A vertex u of a common net, into the set (u < 0: none).  True if it is new.
+__device__ __forceinline__ bool list_insert(unsigned* set, int log, int u) {
+    if (u < 0) return false;
+    const unsigned mask = (1u << log) - 1u;
+    for (unsigned h = (unsigned)u * 0x9E3779B1u >> (32 - log);; h = (h + 1u) & mask) {
+        const unsigned seen = *(volatile unsigned*)(set + h);
+        if (seen == (unsigned)u) return false;
+        if (seen != kListEmpty) continue;
+        const unsigned old = atomicCAS(set + h, kListEmpty, (unsigned)u);
+        if (old == kListEmpty) return true;
+        if (old == (unsigned)u) return false;
+    }
+}
+
+// Append e to list where pred holds (all 32 lanes call; one atomic).
+__device__ __forceinline__ void append_warp(bool pred, int4 e, int4* list, int* count) {
+    const unsigned m = __ballot_sync(kFullMask, pred);
+    if (m == 0u) return;
+    int at = 0;
+    if (lane_id() == 0) at = atomicAdd(count, __popc(m));
+    at = __shfl_sync(kFullMask, at, 0);
+    if (pred) list[at + __popc(m & ((1u << lane_id()) - 1u))] = e;
+}
+
+__global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ Pp,
+                          const d1::Problem<d1::ListView>* __restrict__ Lp, ListArgs a) {
+    extern __shared__ uint4 list_sm[];
+    const Problem& P = *Pp;
+    const d1::Problem<d1::ListView>& L = *Lp;
+    d1::State* st = L.st;
+    const int lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    unsigned* const set = reinterpret_cast<unsigned*>(list_sm) + warp * list_warp_ints(a.log);
+    unsigned* const fresh = set + (1 << a.log);
+    const int fresh_cap = (5 << a.log) / 8;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long gw = (long long)blockIdx.x * wpb + warp, nw = (long long)gridDim.x * wpb;
+    const int self = P.self;
+    unsigned at = 0u, end = 0u;   // this warp's part of the buffer
+    unsigned long long my_h = 0ull;
+    bool full = false;
+    for (long long v0 = gw * a.group; v0 < P.n && !full; v0 += nw * a.group) {
+        const int count = (int)min((long long)a.group, P.n - v0);
+        int4 mine = make_int4(-1, 0, 0, 0);   // the worklist entry of vertex v0 + lane
+        // the group's net lists, and the first 32 nets of the vertex that is
+        // next: loaded while the vertex before it is worked on
+        int my_beg = 0, my_k = 0;
+        if (lane < count) {
+            my_beg = __ldg(P.r_ptr + v0 + lane);
+            my_k = __ldg(P.r_ptr + v0 + lane + 1) - my_beg + self;
+        }
+        auto load_nets = [&](int v, int beg, int k, int j, int& q, int& mb, int& ms) {
+            q = mb = ms = 0;
+            if (j >= k) return;
+            q = vertex_net(P, v, beg, j);
+            mb = __ldg(P.m_ptr + q);
+            ms = __ldg(P.m_ptr + q + 1) - mb + self;
+        };
+        int nq, nmb, nms;
+        load_nets((int)v0, __shfl_sync(kFullMask, my_beg, 0), __shfl_sync(kFullMask, my_k, 0), lane,
+                  nq, nmb, nms);
+        for (int x = 0; x < count; ++x) {
+            const int v = (int)v0 + x;
+            const int beg = __shfl_sync(kFullMask, my_beg, x), k = __shfl_sync(kFullMask, my_k, x);
+            int log = a.log, found = 0;
+            for (int j0 = 0; j0 < k || j0 == 0; j0 += 32) {
+                // 32 nets: lane j holds net j's members' place among all
+                int q = nq, mb = nmb, ms = nms;
+                if (j0 > 0) {
+                    load_nets(v, beg, k, j0 + lane, q, mb, ms);
+                } else if (x + 1 < count) {
+                    load_nets(v + 1, __shfl_sync(kFullMask, my_beg, x + 1),
+                              __shfl_sync(kFullMask, my_k, x + 1), lane, nq, nmb, nms);
+                }
+                int incl = ms;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(kFullMask, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                const int total = __shfl_sync(kFullMask, incl, 31);
+                if (j0 == 0) {
+                    // v's own set: about half full if no member repeats (short
+                    // probes), no larger than needed (it has to be cleared)
+                    if (k <= 32) {
+                        log = kListMinLog;
+                        while (log < a.log && (1 << log) < 2 * total) ++log;
+                    }
+                    for (int s = lane; s < (1 << log) / 4; s += 32)
+                        reinterpret_cast<uint4*>(set)[s] =
+                            make_uint4(kListEmpty, kListEmpty, kListEmpty, kListEmpty);
+                    __syncwarp();
+                }
+                auto insert = [&](int u) {
+                    const bool is_new = list_insert(set, log, u == v ? -1 : u);
+                    const unsigned m = __ballot_sync(kFullMask, is_new);
+                    const int to = found + __popc(m & lt);
+                    if (is_new && to < fresh_cap) fresh[to] = (unsigned)u;
+                    found += __popc(m);
+                };
+                if (total >= 20 * min(32, k - j0)) {
+                    // nets that nearly fill a warp: four nets at a time, 32
+                    // members of each
+                    const int most = (int)__reduce_max_sync(kFullMask, (unsigned)ms);
+                    for (int j = 0; j < min(32, k - j0); j += 4)
+                        for (int m0 = 0; m0 < most; m0 += 32) {
+                            int u[4];
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const int qo = __shfl_sync(kFullMask, q, j + c);
+                                const int bo = __shfl_sync(kFullMask, mb, j + c);
+                                const int so = __shfl_sync(kFullMask, ms, j + c);
+                                const int m = m0 + lane - self;
+                                u[c] = m0 + lane >= so ? -1
+                                       : m < 0 ? qo : __ldg(P.m_idx + bo + m);
+                            }
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) insert(u[c]);
+                        }
+                } else {
+                    // short nets: their members flattened over the lanes
+                    for (int f0 = 0; f0 < total; f0 += 128) {
+                        int u[4];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const int f = f0 + 32 * c + lane;
+                            int o = 0;   // the net of member f
+#pragma unroll
+                            for (int step = 16; step; step >>= 1)
+                                if (__shfl_sync(kFullMask, incl, o + step - 1) <= f) o += step;
+                            const int qo = __shfl_sync(kFullMask, q, o);
+                            const int bo = __shfl_sync(kFullMask, mb, o);
+                            const int m = f - __shfl_sync(kFullMask, incl - ms, o) - self;
+                            u[c] = f >= total ? -1 : m < 0 ? qo : __ldg(P.m_idx + bo + m);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) insert(u[c]);
+                    }
+                }
+            }
+            const int len = found;
+            __syncwarp();
+            if (at + (unsigned)len > end) {
+                const unsigned take = max(a.chunk, (unsigned)len);
+                unsigned long long b = 0ull;
+                if (lane == 0) b = atomicAdd(&P.st->list_next, (unsigned long long)take);
+                b = __shfl_sync(kFullMask, b, 0);
+                if (b + (unsigned long long)len > (unsigned long long)a.cap) {
+                    full = true;   // the call falls back to the net rounds
+                    break;
+                }
+                at = (unsigned)b;
+                end = (unsigned)min(b + take, (unsigned long long)a.cap);
+            }
+            const unsigned long long kv = __ldg(P.key + v);
+            int hi_n = 0, lo_n = 0;
+            int* const front = a.lists + at;
+            int* const back = front + len - 1;
+            const bool staged = len <= fresh_cap;
+            const unsigned* const from = staged ? fresh : set;
+            const int from_n = staged ? len : k == 0 ? 0 : 1 << log;
+            for (int s0 = 0; s0 < from_n; s0 += 128) {
+                unsigned u[4];
+                unsigned long long ku[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    u[c] = s0 + 32 * c + lane < from_n ? from[s0 + 32 * c + lane] : kListEmpty;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    ku[c] = u[c] != kListEmpty ? __ldg(P.key + u[c]) : 0ull;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const bool in = u[c] != kListEmpty;
+                    const bool hi = in && key_priority(ku[c], (int)u[c], kv, v, P.seed);
+                    const unsigned bh = __ballot_sync(kFullMask, hi);
+                    const unsigned bl = __ballot_sync(kFullMask, in && !hi);
+                    if (hi) front[hi_n + __popc(bh & lt)] = (int)u[c];
+                    else if (in) back[-(lo_n + __popc(bl & lt))] = (int)u[c];
+                    hi_n += __popc(bh);
+                    lo_n += __popc(bl);
+                }
+            }
+            if (lane == x) mine = make_int4(v, hi_n, len, (int)at);
+            if (len >= 64)
+                for (int w = lane; w <= len >> 5; w += 32)
+                    L.bmx[(long long)v * L.g.bm_words + w] = 0u;
+            at += (unsigned)len;
+            __syncwarp();
+        }
+        const bool have = mine.x >= 0;
+        if (have) {
+            a.rows[mine.x] = make_int2(mine.w, mine.z);
+            L.col[mine.x] = -1;
+            my_h += (unsigned long long)mine.y;
+        }
+        append_warp(have && mine.y <= L.det_s, mine, L.ws[1], &st->ns[1]);
+        append_warp(have && mine.y > L.det_s, mine, L.wm[1], &st->nm[1]);
+    }
+    my_h = warp_sum(my_h);
+    if (lane == 0 && my_h) atomicAdd(&st->h_first, my_h);
+    if (full && lane == 0) {
+        st->status = d1::ST_LISTS;
+        st->done = 1;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->round = 1;
+        st->t0 = global_ns();
+        if (P.n <= L.mid_w) st->mid = 1;
+        if (L.trace_cap > 0) {
+            L.trace_w[0] = P.n;
+            L.trace_s[0] = __ldg(P.r_ptr + P.n);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // PD2 over every vertex of B (Sec. 3.6): one net problem with both sides.
 // Vertices: the n_cols columns (ids 0..n_cols-1), then the rows (n_cols + i).
 // Nets: the rows (net i, members = its columns), then the columns (net
@@ -1038,19 +1309,113 @@ struct Input {
     int* col;
 };
 
-static pgc_status run_scratch(Context& cx, const Input& in, uint64_t seed, const Opts& o,
+static pgc_status run_scratch(Context& cx, const Input& in, int nnz, uint64_t seed, const Opts& o,
                               cudaStream_t stream, int* rounds, int* num_colors);
 
 // Out of device memory: keep no half-grown scratch (the next call allocates
 // again).
-static pgc_status run(Context& cx, const Input& in, uint64_t seed, const Opts& o,
+static pgc_status run(Context& cx, const Input& in, int nnz, uint64_t seed, const Opts& o,
                       cudaStream_t stream, int* rounds, int* num_colors) {
-    pgc_status s = run_scratch(cx, in, seed, o, stream, rounds, num_colors);
+    pgc_status s = run_scratch(cx, in, nnz, seed, o, stream, rounds, num_colors);
     if (s == PGC_ERR_OOM) cx.release();
     return s;
 }
 
-static pgc_status run_scratch(Context& cx, const Input& in, uint64_t seed, const Opts& o,
+// The coloring as a distance-1 coloring of the conflict graph, once net_init
+// has run and hs holds its sums.  *taken is false when the problem is left to
+// the net rounds: a vertex with too many members for a warp's set, lists that
+// would not fit kListMaxEntries, or no device memory for them.
+static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& hs, uint64_t seed,
+                            const Opts& o, cudaStream_t stream, int* rounds, int* num_colors,
+                            bool* taken) {
+    using E = d1::Engine<d1::ListView>;
+    *taken = false;
+    const int n = in.n;
+    if (hs.members >= 1 << kListMaxLog || hs.pairs > 8 * kListMaxEntries) return PGC_OK;
+    E* eng = d1::engine_for<d1::ListView>(cx.dev.device);
+    std::lock_guard<std::mutex> lk(eng->mu);
+    eng->dev = cx.dev;
+
+    ListArgs a = {};
+    a.log = kListMinLog;
+    while (1 << a.log <= hs.members) ++a.log;
+    const int block = 256, wpb = block / 32;
+    const size_t smem = (size_t)wpb * list_warp_ints(a.log) * 4;
+    if (smem > 48 * 1024)
+        PGC_CUDA(cudaFuncSetAttribute(net_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
+    int per_sm = 0;
+    PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, net_lists, block, smem));
+    const int grid = cx.dev.num_sms * std::max(1, per_sm);
+    const long long warps = (long long)grid * wpb;
+    // A warp takes 8 of the longest rows at a time from the counter, or each
+    // row by itself when there are few per warp.  A part's rest is left when
+    // the next row does not fit: less than a row in 8, and a part per warp.
+    a.group = (int)std::max<long long>(1, std::min<long long>(32, n / warps));
+    a.chunk = n >= 8 * warps ? 8u * (unsigned)hs.members : 0u;
+    unsigned long long cap = hs.pairs;
+    if (a.chunk) cap += hs.pairs / 7 + (unsigned long long)warps * (a.chunk + hs.members);
+    a.cap = (unsigned)std::max<unsigned long long>(1, std::min(cap, kListMaxEntries));
+
+    const int bm_words = (hs.members >> 5) + 1;
+    const d1::ScratchSizes z = d1::scratch_sizes(n, 0);
+    pgc_status s = PGC_OK;
+    auto need = [&](DevBuf& b, size_t bytes) {
+        if (s == PGC_OK) s = b.ensure(bytes);
+    };
+    need(eng->deg, (size_t)n * sizeof(int2));   // the rows
+    need(eng->hlen, z.hlen);
+    need(eng->hadj, (size_t)a.cap * 4);
+    need(eng->bm0, z.bm0);
+    need(eng->bmx, (size_t)n * bm_words * 4);
+    need(eng->live, z.live);
+    need(eng->ws, z.list);
+    need(eng->wm, z.list);
+    need(eng->wl, z.list);
+    need(eng->pushq, ((size_t)n + a.cap / d1::kPushItem + 1) * sizeof(int2));
+    if (s == PGC_ERR_OOM) {
+        eng->release();
+        return PGC_OK;
+    }
+    if (s != PGC_OK) return s;
+    a.rows = eng->deg.as<int2>();
+    a.lists = eng->hadj.as<int>();
+    d1::Scratch sc = {};
+    sc.hlen = eng->hlen.as<int>();
+    sc.hadj = a.lists;
+    sc.bm0 = eng->bm0.as<unsigned long long>();
+    sc.bmx = eng->bmx.as<unsigned>();
+    sc.live = eng->live.as<unsigned>();
+    sc.ws = eng->ws.as<int4>();
+    sc.wm = eng->wm.as<int4>();
+    sc.wl = eng->wl.as<int4>();
+    sc.pushq = eng->pushq.as<int2>();
+    d1::ListView view{a.rows, a.lists, in.r_ptr, bm_words};
+    Opts lo = o;
+    lo.mid_degree = kListMid;
+    lo.hub_degree = 1 << kListMaxLog;
+    const Problem* dP = cx.problem.as<Problem>();
+    const E::Setup setup = [&](const d1::Problem<d1::ListView>* dL) -> pgc_status {
+        PGC_CUDA(cudaMemsetAsync(eng->live.ptr, 0xff, z.live, stream));
+        PGC_CUDA(cudaMemsetAsync(eng->bm0.ptr, 0, z.bm0, stream));
+        net_lists<<<grid, block, smem, stream>>>(dP, dL, a);
+        PGC_CUDA(cudaGetLastError());
+        return PGC_OK;
+    };
+    s = eng->launch(sc, view, n, nnz, in.col, nullptr, nullptr, seed, lo, stream, nullptr, &setup);
+    if (s == PGC_OK) PGC_CUDA(cudaStreamSynchronize(stream));
+    if (s == PGC_ERR_OOM) {
+        PGC_CUDA(cudaStreamSynchronize(stream));
+        eng->release();
+        return PGC_OK;
+    }
+    if (s != PGC_OK) return s;
+    if (eng->h_state.as<d1::State>()->status == d1::ST_LISTS) return PGC_OK;
+    *taken = true;
+    return eng->finish(lo, rounds, num_colors);
+}
+
+static pgc_status run_scratch(Context& cx, const Input& in, int nnz, uint64_t seed, const Opts& o,
                               cudaStream_t stream, int* rounds, int* num_colors) {
     const int n = in.n;
     if (pgc_status s = cx.key.ensure((size_t)n * 8)) return s;
@@ -1116,6 +1481,15 @@ static pgc_status run_scratch(Context& cx, const Input& in, uint64_t seed, const
     if (pgc_status s = kt.end()) return s;
     PGC_CUDA(cudaMemcpyAsync(hs, cx.state.ptr, sizeof(State), cudaMemcpyDeviceToHost, stream));
     PGC_CUDA(cudaStreamSynchronize(stream));
+    bool taken = false;
+    if (pgc_status s = run_lists(cx, in, nnz, *hs, seed, o, stream, rounds, num_colors, &taken)) {
+        kt.destroy();
+        return s;
+    }
+    if (taken) {
+        kt.destroy();
+        return PGC_OK;
+    }
     const long long need = (long long)hs->bound + 1;   // a first-fit color is <= |S(v)| + 1
     const int windows = (int)std::min<long long>(kMaxWindows, (need + 63) / 64);
     hp->windows = std::max(1, windows);
@@ -1407,7 +1781,7 @@ static pgc_status color(int kind, int32_t n_rows, int32_t n_cols, const int32_t*
         if (pgc_status s = cx->stage_col.ensure((size_t)n * 4)) return s;
         in.col = cx->stage_col.as<int>();
     }
-    pgc_status s = run(*cx, in, seed, o, stream, rounds, num_colors);
+    pgc_status s = run(*cx, in, nnz, seed, o, stream, rounds, num_colors);
     if (s != PGC_OK) return s;
     if (host_col) {
         PGC_CUDA(cudaMemcpyAsync(colors, in.col, (size_t)n * 4, cudaMemcpyDeviceToHost, stream));

@@ -352,6 +352,7 @@ pgc_status pgc_server_create(size_t hbm_budget_bytes, int32_t max_active, pgc_se
             cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
             cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
             sl.d1e.dev.device = S.device;
+            sl.d1e.shares_gpu = true;
             cudaDeviceGetAttribute(&sl.d1e.dev.num_sms, cudaDevAttrMultiProcessorCount, S.device);
         }
         S.engine = std::thread(pgc::serve::engine_loop, &S);
