@@ -221,7 +221,7 @@ static pgc_status color_batch(int32_t G, const int64_t* vtx_off, const int64_t* 
                                                                  B.gid.as<int>(), d_gr, d_gc);
     PGC_CUDA(cudaGetLastError());
     BatchView view{(const long long*)d_vo, (const long long*)d_no, (const int*)d_rp,
-                   (const int*)d_ci, B.gid.as<int>()};
+                   (const int*)d_ci, B.gid.as<int>(), NNZ <= (long long)UINT32_MAX ? 1 : 0};
 
     int rounds = 0, ncolors = 0;
     if (o.flags & PGC_AUTOTUNE) {

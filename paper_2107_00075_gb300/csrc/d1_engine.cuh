@@ -83,12 +83,14 @@ struct SingleView {
         d = __ldg(rp + v + 1) - r0;
     }
     __device__ __forceinline__ int nbr(long long e, int) const { return __ldg(ci + e); }
-    // start of v's row relative to its graph, and the absolute start from it
+    // row start as entries hold it, and degree
     __device__ __forceinline__ void local_row(int v, int, int& r0, int& d) const {
         r0 = __ldg(rp + v);
         d = __ldg(rp + v + 1) - r0;
     }
-    __device__ __forceinline__ long long begin(int, int r0) const { return r0; }
+    // absolute start of v's row from an entry's row start
+    __device__ __forceinline__ int begin(int, int r0) const { return r0; }
+    using Off = int;
     // first overflow word of v, whose row starts at b: v owns deg/32 + 1 words
     __device__ __forceinline__ long long bm(int v, long long b) const { return (b >> 5) + v; }
     // the degree in v's priority, from its row length d
@@ -104,6 +106,8 @@ struct BatchView {
     const int* rp;
     const int* ci;
     const int* gid;   // graph of each global vertex
+    int absolute;     // entries hold absolute row starts (fewer than 2^32 entries in the
+                      // batch): two dependent loads less per entry
     __device__ __forceinline__ int graph(int v) const { return __ldg(gid + v); }
     __device__ __forceinline__ int base(int g) const { return (int)__ldg(vtx_off + g); }
     __device__ __forceinline__ void row(int v, int g, long long& b, int& d) const {
@@ -117,10 +121,12 @@ struct BatchView {
     __device__ __forceinline__ void local_row(int v, int g, int& r0, int& d) const {
         r0 = __ldg(rp + v + g);
         d = __ldg(rp + v + g + 1) - r0;
+        if (absolute) r0 = (int)(unsigned)(__ldg(nnz_off + g) + r0);
     }
-    __device__ __forceinline__ long long begin(int g, int r0) const {
-        return __ldg(nnz_off + g) + r0;
+    __device__ __forceinline__ long long begin(int v, int r0) const {
+        return absolute ? (long long)(unsigned)r0 : __ldg(nnz_off + graph(v)) + r0;
     }
+    using Off = long long;
     __device__ __forceinline__ long long bm(int v, long long b) const { return (b >> 5) + v; }
     __device__ __forceinline__ int degree(int, int d) const { return d; }
     static constexpr bool kSetup = true;
@@ -143,7 +149,8 @@ struct ListView {
         d = x.y;
     }
     __device__ __forceinline__ int nbr(long long e, int) const { return __ldg(ci + e); }
-    __device__ __forceinline__ long long begin(int, int r0) const { return r0; }
+    __device__ __forceinline__ int begin(int, int r0) const { return r0; }
+    using Off = int;
     __device__ __forceinline__ long long bm(int v, long long) const {
         return (long long)v * bm_words;
     }
@@ -184,12 +191,14 @@ struct Hot {
     int push_cnt;     // push work items queued this round
     int max_color;
     int stop;         // mid loop: round in which the time limit had passed (0: none)
+    int pend;         // round 1's queued pushes still wait (setup queues them)
     __host__ __device__ int count(int p) const { return ns[p] + nm[p] + nl[p]; }
 };
 
 struct State : Hot {
     int status;       // ST_*
     int bs, bm, bc;   // setup: vertices (S, M) and items (C) per degree class
+    int lists_full;   // ListView: the lists did not fit their buffer
     unsigned blocks_done;
     int bar_timeout;            // mid loop: a barrier wait gave up
     unsigned long long s_next;  // sum of degrees of the next worklist
@@ -198,10 +207,7 @@ struct State : Hot {
     unsigned long long t0;      // globaltimer at start
     int core_k;       // core phase: vertices of the induced subgraph
     int core_par;     // core phase: parity whose worklist buffers hold its arrays
-    // mid loop grid barrier, arrivals and generation, a line each: the pollers
-    // of one do not delay the arrivals at the other
-    alignas(128) unsigned bar_count;
-    alignas(128) unsigned bar_gen;
+    alignas(128) unsigned bar_count;   // mid loop grid barrier: arrivals, a line of its own
 };
 
 template <class V>
@@ -383,7 +389,7 @@ __global__ void d1_classify(const Problem<V>* __restrict__ Pp) {
             const int v = (int)i;
             const int g = P.g.graph(v);
             P.g.local_row(v, g, r0, d);
-            const long long b = P.g.begin(g, r0);
+            const long long b = P.g.begin(v, r0);
             P.deg[v] = d;
             P.col[v] = P.async_mode ? 0 : -1;
             if (P.prio_mode) P.prio[v] = P.prio_mode == 1 ? d : 0;
@@ -469,7 +475,7 @@ __global__ void __maxnreg__(40) d1_build(const Problem<V>* __restrict__ Pp, int 
         const int v = ent.x, d = ent.z;
         if (v < lo || v >= hi) continue;
         const int g = P.g.graph(v), base = P.g.base(g);
-        const long long beg = P.g.begin(g, ent.w);
+        const long long beg = P.g.begin(v, ent.w);
         const uint64_t hv = prio_hash(seed, (uint32_t)(v - base));
         int pos = 0;
         for (int b0 = 0; b0 < d; b0 += 32) {
@@ -497,7 +503,7 @@ __global__ void __maxnreg__(40) d1_build(const Problem<V>* __restrict__ Pp, int 
         const int v = ent.x, d = ent.z;
         if (v < lo || v >= hi) continue;
         const int g = P.g.graph(v), base = P.g.base(g);
-        const long long beg = P.g.begin(g, ent.w);
+        const long long beg = P.g.begin(v, ent.w);
         const uint64_t hv = prio_hash(seed, (uint32_t)(v - base));
         int pos = 0;
         for (int e0 = 0; e0 < d; e0 += 4) {
@@ -519,33 +525,6 @@ __global__ void __maxnreg__(40) d1_build(const Problem<V>* __restrict__ Pp, int 
 }
 
 // ---------------------------------------------------------------------------
-// setup 3: round-1 worklists by |H(v)|
-// ---------------------------------------------------------------------------
-template <class V>
-__global__ void d1_tier(const Problem<V>* __restrict__ Pp) {
-    __shared__ int s_n[2][33];
-    const Problem<V>& P = *Pp;
-    State* st = P.st;
-    const int n = P.n;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
-        const long long i = base + threadIdx.x;
-        const bool valid = i < n;
-        int4 e = make_int4((int)i, 0, 0, 0);   // {v, |H(v)|, deg(v), local row start}
-        if (valid) {
-            int r0, d;
-            P.g.local_row((int)i, P.g.graph((int)i), r0, d);
-            e = make_int4((int)i, P.hlen[i], d, r0);
-        }
-        block_append(valid && e.y <= P.det_s, valid && e.y > P.det_s && e.y <= P.det_m, e,
-                     P.ws[1], &st->ns[1], P.wm[1], &st->nm[1], s_n);
-        if (valid && e.y > P.det_m) P.wl[1][atomicAdd(&st->nl[1], 1)] = e;
-    }
-    // a graph of at most mid_w vertices runs all its rounds in the mid loop
-    if (blockIdx.x == 0 && threadIdx.x == 0 && n <= P.mid_w) st->mid = 1;
-}
-
-// ---------------------------------------------------------------------------
 // assign: first fit from the forbidden-color set
 // ---------------------------------------------------------------------------
 // First fit for worklist entry e = {v, |H(v)|, deg(v), local row start}.
@@ -561,8 +540,7 @@ __device__ __forceinline__ int first_fit(const Problem<V>& P, int4 e, int tp,
     if (w0 != ~0ull) {
         t = __ffsll((long long)~w0);
     } else {   // colors 1..64 all taken: deg(v) >= 64, scan the overflow bitmap
-        const int g = P.g.graph(v);
-        const long long b = P.g.begin(g, e.w);
+        const long long b = P.g.begin(v, e.w);
         const int words = (e.z >> 5) + 1;
         const unsigned* w = P.bmx + P.g.bm(v, b);
         // four words per step, from the word that holds the previous color
@@ -596,8 +574,8 @@ __device__ __forceinline__ int first_fit(const Problem<V>& P, int4 e, int tp,
 }
 
 template <class V>
-__device__ __forceinline__ void assign_phase(const Problem<V>& P, const Hot& h) {
-    const int cp = h.round & 1;
+__device__ __forceinline__ void assign_phase(const Problem<V>& P, const Hot& h, int r) {
+    const int cp = r & 1;
     const int n0 = h.ns[cp], n1 = h.nm[cp], n2 = h.nl[cp];
     const long long total = (long long)n0 + n1 + n2;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -650,7 +628,7 @@ __device__ __forceinline__ void assign_async_phase(const Problem<V>& P, const Ho
                      : (i < n0 + n1 ? P.wm[cp][i - n0] : P.wl[cp][i - n0 - n1]);
         const int v = e.x, d = e.z;
         const int g = P.g.graph(v), base = P.g.base(g);
-        const long long beg = P.g.begin(g, e.w);
+        const long long beg = P.g.begin(v, e.w);
         int t = 0;
         for (int w = 0; t == 0; ++w) {
             unsigned long long f = 0ull;
@@ -693,20 +671,20 @@ __global__ void d1_assign(const Problem<V>* __restrict__ Pp, State* st,
         st->push_cnt = 0;   // the previous round's push kernel has finished
     }
     if (P.async_mode) assign_async_phase(P, ctx.h);
-    else assign_phase(P, ctx.h);
+    else assign_phase(P, ctx.h, ctx.h.round);
 }
 
 // ---------------------------------------------------------------------------
 // detect + commit + compact + inline push (+ round control in the last block)
 // ---------------------------------------------------------------------------
 // End of round r: record the trace, decide whether to go on, set up round
-// r+1.  Returns 1 when the coloring is finished (or has failed).
+// r+1.  cur: the round's worklist.  Returns 1 when the coloring is finished (or
+// has failed).
 template <class V>
-__device__ int round_decide(const Problem<V>& P) {
+__device__ int round_decide(const Problem<V>& P, long long cur) {
     State* st = P.st;
     const int r = st->round;
     const int cp = r & 1, np = cp ^ 1;
-    const long long cur = (long long)st->ns[cp] + st->nm[cp] + st->nl[cp];
     const long long nxt = (long long)*(volatile int*)&st->ns[np] + *(volatile int*)&st->nm[np] +
                           *(volatile int*)&st->nl[np];
     if (r < P.trace_cap) {
@@ -747,7 +725,8 @@ __device__ int round_decide(const Problem<V>& P) {
 // remaining rounds go to the mid loop.
 template <class V>
 __device__ void round_control(const Problem<V>& P, cudaGraphConditionalHandle h, int use_cond) {
-    const int done = round_decide(P);
+    const int cp = P.st->round & 1;
+    const int done = round_decide(P, (long long)P.st->ns[cp] + P.st->nm[cp] + P.st->nl[cp]);
     if (use_cond) cudaGraphSetConditional(h, (done || P.st->mid) ? 0u : 1u);
 }
 
@@ -842,6 +821,121 @@ __device__ __forceinline__ bool deal_any(const Deal& d, int rank, const unsigned
     return (w >> (from & 31) & (kFullMask >> (32 - (1 << d.log)))) != 0u;
 }
 
+// ---------------------------------------------------------------------------
+// setup 3: worklists by |H(v)|, and round 1
+// ---------------------------------------------------------------------------
+// In round 1 every vertex holds color 1, so v wins exactly when H(v) is empty,
+// and no list is read: the winners commit here and the others are round 2's
+// worklists (a pass over all entries less: 5.0 of 52 ms for the 4096-graph
+// batch).  None of a winner's neighbors wins, so its pushes ask nobody.  With
+// PGC_ASYNC or a round-varying priority round 1 is a round like any other.
+template <class V>
+__device__ __forceinline__ bool round1_in_setup(const Problem<V>& P) {
+    return !P.async_mode && !P.prio_mode;
+}
+
+// The last block to finish ends round 1 (all threads call).
+template <class V>
+__device__ __forceinline__ void end_round1(const Problem<V>& P, State* st) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&st->blocks_done, 1u) == gridDim.x - 1;
+        if (s_last) {
+            __threadfence();
+            st->max_color = 1;
+            st->pend = 1;
+            round_decide(P, P.n);
+            if (*(volatile int*)&st->lists_full) {
+                st->status = ST_LISTS;
+                st->done = 1;
+                st->mid = 0;
+            }
+        }
+    }
+}
+
+template <class V>
+__global__ void d1_tier(const Problem<V>* __restrict__ Pp, State* st) {
+    __shared__ int s_n[2][33];
+    __shared__ unsigned char s_slot[32][32];
+    __shared__ Ctx<V> ctx;
+    const Problem<V>& P = enter(ctx, Pp, st);
+    const int n = P.n, lane = lane_id();
+    const bool first = round1_in_setup(P), traced = P.trace_cap > 0;
+    const int p = first ? 0 : 1;   // parity of the worklists made here
+    unsigned char* const slot = s_slot[threadIdx.x >> 5];
+    unsigned long long sum_s = 0ull, sum_h = 0ull;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
+        const long long i = base + threadIdx.x;
+        const bool valid = i < n;
+        int4 e = make_int4((int)i, 0, 0, 0);   // {v, |H(v)|, deg(v), row start}
+        if (valid) {
+            int r0, d;
+            P.g.local_row((int)i, P.g.graph((int)i), r0, d);
+            e = make_int4((int)i, P.hlen[i], d, r0);
+        }
+        const bool win = valid && first && e.y == 0, go_on = valid && !win;
+        block_append(go_on && e.y <= P.det_s, go_on && e.y > P.det_s && e.y <= P.det_m, e, P.ws[p],
+                     &st->ns[p], P.wm[p], &st->nm[p], s_n);
+        if (go_on && e.y > P.det_m) P.wl[p][atomicAdd(&st->nl[p], 1)] = e;
+        if (!first) continue;
+        if (traced && go_on) {
+            sum_s += (unsigned long long)e.z;
+            sum_h += (unsigned long long)e.y;
+        }
+        const unsigned wins = __ballot_sync(kFullMask, win);
+        if (!wins) continue;
+        int g = 0;
+        if (win) {
+            P.col[e.x] = 1;
+            if (P.g_rounds != nullptr) g = P.g.graph(e.x);
+        }
+        if (lane == __ffs(wins) - 1) P.live[e.x >> 5] &= ~wins;   // 32 vertices, one word
+        if (P.g_rounds != nullptr) graph_max(P.g_colors, win, g, 1);
+        queue_push(P, win && e.z > kInlinePush, e.x, e.z);
+        const long long beg = win ? P.g.begin(e.x, e.w) : 0;
+        const int nb = win ? P.g.base(P.g.graph(e.x)) : 0;
+        unsigned open = __ballot_sync(kFullMask, win && e.z > 0 && e.z <= kInlinePush);
+        for (int pos = 0; open;) {   // the neighbors' bit for color 1
+            const Deal deal = deal_rows(open, slot);
+            const int per = 1 << deal.log;
+            int u[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int src = deal_lane(deal, slot, j), from = src < 0 ? lane : src;
+                const int x = pos + ((32 * j + lane) & (per - 1));
+                const int len = __shfl_sync(kFullMask, e.z, from);
+                const int v = __shfl_sync(kFullMask, e.x, from);
+                const int ub = __shfl_sync(kFullMask, nb, from);
+                const long long b = __shfl_sync(kFullMask, beg, from);
+                u[j] = src >= 0 && x < len ? P.g.nbr(b + x, ub) : -1;
+                if (u[j] == v) u[j] = -1;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (u[j] >= 0) atomicOr(P.bm0 + u[j], 1ull);
+            pos += per;
+            open = __ballot_sync(kFullMask, (open >> lane & 1u) && pos < e.z);
+        }
+    }
+    if (first) {
+        if (traced) {
+            sum_s = warp_sum(sum_s);
+            sum_h = warp_sum(sum_h);
+            if (lane == 0 && (sum_s || sum_h)) {
+                atomicAdd(&st->s_next, sum_s);
+                atomicAdd(&st->h_next, sum_h);
+            }
+        }
+        end_round1(P, st);
+    } else if (blockIdx.x == 0 && threadIdx.x == 0 && n <= P.mid_w) {
+        st->mid = 1;   // all rounds in the mid loop
+    }
+}
+
 // One tier's worklist: conflict search, commit, inline push and re-append.
 //
 // A warp takes up to 32 worklist vertices and searches their lists together:
@@ -871,32 +965,31 @@ __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* lis
     const int* __restrict__ ha = P.hadj;
     int* const col = P.col;
     const bool batch = P.g_rounds != nullptr, traced = P.trace_cap > 0;
-    // round 1: every vertex holds tentative color 1, so v loses exactly when
-    // H(v) is not empty -- no list needs to be read
-    const bool first = r == 1 && !P.async_mode && !DYN;
     const int lane = lane_id(), wpb = blockDim.x >> 5;
     const long long gw = (long long)blockIdx.x * wpb + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * wpb;
     int take = 32;   // vertices per warp: the smallest power of two that is one pass
     while (take > 1 && (take >> 1) * nw >= n) take >>= 1;
+    using Off = typename V::Off;
+    int4 ahead = make_int4(0, 0, 0, 0);   // the next vertex's entry, one step ahead
+    if (lane < take && gw * take + lane < n) ahead = list[gw * take + lane];
     for (long long i0 = gw * take; i0 < n; i0 += nw * take) {
         const long long i = i0 + lane;
         const bool valid = lane < take && i < n;
-        int4 ent = make_int4(0, 0, 0, 0);
-        int g = 0, t = 0;
-        long long beg = 0;
+        const int4 ent = ahead;
+        if (i + nw * take < n && lane < take) ahead = list[i + nw * take];
+        int t = 0;
+        Off beg = 0;
         MeOf<DYN> me{};
         if (valid) {
-            ent = list[i];
-            g = P.g.graph(ent.x);
-            beg = P.g.begin(g, ent.w);
+            beg = P.g.begin(ent.x, ent.w);
             t = -col[ent.x];
-            if constexpr (DYN) me = round_me(P, ent.x, g);
+            if constexpr (DYN) me = round_me(P, ent.x, P.g.graph(ent.x));
         }
         const int v = ent.x, hl = ent.y, d = ent.z;
-        bool lose = valid && first && hl > 0;
+        bool lose = false;
         int pos = 0;   // entries read of every list still open
-        unsigned open = __ballot_sync(kFullMask, valid && !first && hl > 0);
+        unsigned open = __ballot_sync(kFullMask, valid && hl > 0);
         while (open) {   // warp-uniform
             const Deal deal = deal_rows(open, slot);
             const int per = 1 << deal.log;
@@ -907,7 +1000,7 @@ __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* lis
                 const int src = deal_lane(deal, slot, j), from = src < 0 ? lane : src;
                 const int x = pos + ((32 * j + lane) & (per - 1));
                 const int len = __shfl_sync(kFullMask, hl, from);
-                const long long b = __shfl_sync(kFullMask, beg, from);
+                const Off b = __shfl_sync(kFullMask, beg, from);
                 ut[j] = __shfl_sync(kFullMask, t, from);
                 if constexpr (DYN) {
                     ume[j].v = __shfl_sync(kFullMask, me.v, from);
@@ -932,6 +1025,7 @@ __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* lis
             open = __ballot_sync(kFullMask, mine);
         }
         const bool win = valid && !lose;
+        const int g = batch && win ? P.g.graph(v) : 0;
         if (lose) {
             sum.s += (unsigned long long)(V::kSetup ? d : traced ? P.g.degree(v, d) : 0);
             sum.h += (unsigned long long)hl;
@@ -963,7 +1057,7 @@ __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* lis
                     const int x =
                         __shfl_sync(kFullMask, pos, from[j]) + ((32 * j + lane) & (per - 1));
                     const int len = __shfl_sync(kFullMask, d, from[j]);
-                    const long long b = __shfl_sync(kFullMask, beg, from[j]);
+                    const Off b = __shfl_sync(kFullMask, beg, from[j]);
                     const int uv = __shfl_sync(kFullMask, v, from[j]);
                     const int ug = __shfl_sync(kFullMask, g, from[j]);
                     u[j] = src >= 0 && x < len ? P.g.nbr(b + x, P.g.base(ug)) : -1;
@@ -994,11 +1088,12 @@ __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* lis
 // lists then hold every neighbor, and a neighbor holding v's color must also
 // beat v this round.
 template <class V, bool DYN>
-__device__ __forceinline__ void detect_phase(const Problem<V>& P, const Hot& hot, int* smem) {
+__device__ __forceinline__ void detect_phase(const Problem<V>& P, const Hot& hot, int r,
+                                             int* smem) {
     __shared__ unsigned char s_slot[32][32];
     __shared__ int s_n[2][33], s_max;
     State* st = P.st;
-    const int r = hot.round, cp = r & 1, np = cp ^ 1;
+    const int cp = r & 1, np = cp ^ 1;
     const int nS = hot.ns[cp], nM = hot.nm[cp], nL = hot.nl[cp];
     const int* __restrict__ ha = P.hadj;
     int* col = P.col;
@@ -1008,7 +1103,6 @@ __device__ __forceinline__ void detect_phase(const Problem<V>& P, const Hot& hot
     // losers keep their entry and tier: appended by source index
     IdxAppend app_s = {smem + warp * 2 * kIdxSlots, 0};
     IdxAppend app_m = {smem + warp * 2 * kIdxSlots + kIdxSlots, 0};
-    const bool first = r == 1 && !P.async_mode && !DYN;
 
     // --- L tier: one block per vertex (static assignment), four entries per
     // thread and step ---
@@ -1016,12 +1110,12 @@ __device__ __forceinline__ void detect_phase(const Problem<V>& P, const Hot& hot
         const int4 ent = P.wl[cp][i];
         const int v = ent.x, hl = ent.y, d = ent.z;
         const int g = P.g.graph(v);
-        const long long beg = P.g.begin(g, ent.w);
+        const long long beg = P.g.begin(v, ent.w);
         const int t = -col[v];
         MeOf<DYN> me{};
         if constexpr (DYN) me = round_me(P, v, g);
-        bool lose = first && hl > 0;
-        for (int b0 = 0; !first && b0 < hl && !lose; b0 += 4 * blockDim.x) {
+        bool lose = false;
+        for (int b0 = 0; b0 < hl && !lose; b0 += 4 * blockDim.x) {
             int u[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -1101,7 +1195,7 @@ __global__ void __maxnreg__(64) d1_detect(const Problem<V>* __restrict__ Pp, Sta
     __shared__ Ctx<V> ctx;
     const Problem<V>& P = enter(ctx, Pp, st);
     if (ctx.h.mid || ctx.h.done) return;   // handed over before round 1, or no lists
-    detect_phase<V, DYN>(P, ctx.h, smem);
+    detect_phase<V, DYN>(P, ctx.h, ctx.h.round, smem);
 
     // --- last block runs the round control ---
     __shared__ int s_last;
@@ -1164,9 +1258,15 @@ __device__ __forceinline__ void reset_next_worklist(const Problem<V>& P, const H
 }
 
 template <class V>
-__global__ void d1_push(const Problem<V>* __restrict__ Pp, State* st) {
+__global__ void d1_push(const Problem<V>* __restrict__ Pp, State* st,
+                        cudaGraphConditionalHandle h, int use_cond) {
     __shared__ Ctx<V> ctx;
     const Problem<V>& P = enter(ctx, Pp, st);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->pend = 0;
+        // before the loop: round 1 has ended, does another one follow?
+        if (use_cond) cudaGraphSetConditional(h, ctx.h.done || ctx.h.mid ? 0u : 1u);
+    }
     push_phase(P, ctx.h.push_cnt);
     if (P.async_mode) reset_next_worklist(P, ctx.h);
 }
@@ -1175,52 +1275,45 @@ __global__ void d1_push(const Problem<V>* __restrict__ Pp, State* st) {
 // mid loop: the rounds of a worklist that does not fill the GPU
 // ---------------------------------------------------------------------------
 // Grid-wide barrier for a cooperative launch (all blocks co-resident), then
-// the block's copy of the counters, for round r (the state's own round moves
-// on at the end of the kernel).  A wait that exceeds max_polls polls (2^22:
-// about a second) gives up, records the failure and lets the kernel return
-// with an error.
-__device__ __forceinline__ bool grid_barrier(State* st, Hot& h, unsigned& gen, unsigned max_polls,
-                                             int r) {
+// the block's copy of the counters.  Arrivals only count up and everyone polls
+// the count itself, so nobody waits for an atomic's answer or for a second
+// word to be written.  `phase`: barriers passed so far.  A wait that exceeds
+// max_polls polls (2^22: about a second) gives up, records the failure and
+// lets the kernel return with an error.
+__device__ __forceinline__ bool grid_barrier(State* st, Hot& h, unsigned& phase,
+                                             unsigned max_polls) {
     __shared__ int s_ok;
     __syncthreads();
+    ++phase;
     if (threadIdx.x < 32) {
         if (threadIdx.x == 0) {
+            const unsigned target = phase * gridDim.x;
             int ok = 1;
-            unsigned arrived;
-            asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;"
-                         : "=r"(arrived) : "l"(&st->bar_count) : "memory");
-            if (arrived == gridDim.x - 1) {
-                asm volatile("st.relaxed.gpu.u32 [%0], 0;" ::"l"(&st->bar_count) : "memory");
-                asm volatile("red.release.gpu.add.u32 [%0], 1;" ::"l"(&st->bar_gen) : "memory");
-            } else {
-                unsigned polls = 0, now;
-                for (;;) {
-                    asm volatile("ld.acquire.gpu.u32 %0, [%1];"
-                                 : "=r"(now) : "l"(&st->bar_gen) : "memory");
-                    if (now != gen) break;
-                    ++polls;
-                    if (polls > max_polls || ((polls & 15u) == 0u && *(volatile int*)&st->bar_timeout)) {
-                        atomicExch(&st->bar_timeout, 1);
-                        ok = 0;
-                        break;
-                    }
-                    if (polls > 64u) __nanosleep(64);
+            asm volatile("red.release.gpu.add.u32 [%0], 1;" ::"l"(&st->bar_count) : "memory");
+            unsigned polls = 0, now;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.u32 %0, [%1];"
+                             : "=r"(now) : "l"(&st->bar_count) : "memory");
+                if (now >= target) break;
+                ++polls;
+                if (polls > max_polls || ((polls & 15u) == 0u && *(volatile int*)&st->bar_timeout)) {
+                    atomicExch(&st->bar_timeout, 1);
+                    ok = 0;
+                    break;
                 }
+                if (polls > 64u) __nanosleep(64);
             }
             s_ok = ok;
         }
         __syncwarp();
         read_hot(h, st);
-        __syncwarp();
-        if (threadIdx.x == 0) h.round = r;
     }
-    ++gen;
     __syncthreads();
     return s_ok != 0;
 }
 
 constexpr int kMidMax = 65536;     // worklists up to this size
-constexpr int kMidThreads = 1024;
+constexpr int kCoreRounds = 8;    // core phase: at this pace, rounds ahead
 constexpr int kMidShared = 8;      // blocks when several colorings share the GPU (the server) ...
 constexpr int kMidSharedMax = 16384;  // ... and their worklists
 
@@ -1243,9 +1336,14 @@ constexpr int kMidSharedMax = 16384;  // ... and their worklists
 // A server colors on many streams: 8 blocks per request leave the SMs to the
 // others (32 requests: 38.7 ms with a block per SM, 22.7 with 8 blocks up to
 // 8,192 vertices, 20.9 up to 16,384).
-template <class V, bool DYN = false>
-__global__ void __launch_bounds__(kMidThreads, 1) d1_mid(const Problem<V>* __restrict__ Pp,
-                                                         State* st) {
+//
+// T threads per block: 1024 for worklists that come from the launched rounds
+// (R-MAT 24 27.8 ms against 29.1 with 512), 512 for problems that are small
+// from the start and for round-varying priorities, whose code then does not
+// spill (PD2 40K x 10K 1.02 -> 0.97 ms, R-MAT 18 with the dynamic degree 4.44
+// -> 4.13).
+template <class V, bool DYN, int T>
+__global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp, State* st) {
     extern __shared__ int smem[];
     __shared__ Ctx<V> ctx;
     const Problem<V>& P = enter(ctx, Pp, st);
@@ -1257,11 +1355,16 @@ __global__ void __launch_bounds__(kMidThreads, 1) d1_mid(const Problem<V>* __res
         const unsigned long long t_end = global_ns() + P.slow_ns;
         while (global_ns() < t_end) __nanosleep(1000);
     }
-    unsigned gen = 0u;
-    auto barrier = [&](int round) { return grid_barrier(st, h, gen, P.bar_polls, round); };
+    unsigned phase = 0u;
+    auto barrier = [&] { return grid_barrier(st, h, phase, P.bar_polls); };
     int r = h.round, cur = h.count(r & 1), status = ST_OK, done = 0, tail = 0;
     const unsigned long long t0 = lead ? st->t0 : 0ull;
-    for (;;) {
+    bool ok = true;
+    if (h.pend && h.push_cnt > 0) {   // round 1's
+        push_phase(P, h.push_cnt);
+        ok = barrier();
+    }
+    while (ok) {
         const int np = (r & 1) ^ 1;
         if (lead) {
             st->push_cnt = 0;
@@ -1271,10 +1374,10 @@ __global__ void __launch_bounds__(kMidThreads, 1) d1_mid(const Problem<V>* __res
             // the timer is slow to read: every eighth round
             if ((r & 7) == 0 && global_ns() - t0 > P.timeout_ns && st->stop == 0) st->stop = r;
         }
-        if (r > 1) assign_phase(P, h);
-        if (!barrier(r)) break;
-        detect_phase<V, DYN>(P, h, smem);
-        if (!barrier(r)) break;
+        if (!DYN || r > 1) assign_phase(P, h, r);
+        if (!barrier()) break;
+        detect_phase<V, DYN>(P, h, r, smem);
+        if (!barrier()) break;
         const int nxt = h.count(np), pushes = h.push_cnt;
         if (lead && P.trace_cap > 0) {
             if (r < P.trace_cap) {
@@ -1289,20 +1392,12 @@ __global__ void __launch_bounds__(kMidThreads, 1) d1_mid(const Problem<V>* __res
         else if (r >= P.max_rounds) status = ST_MAX_ROUNDS;
         else if (h.stop > 0 && h.stop <= r) status = ST_TIMEOUT;
         if (done || status != ST_OK) break;
-        tail = nxt <= P.tail_w && (long long)(cur - nxt) * 8 < nxt;
+        tail = nxt <= P.tail_w && (long long)(cur - nxt) * kCoreRounds < nxt;
         cur = nxt;
         ++r;
         if (pushes > 0) push_phase(P, pushes);
         if (tail) break;
-        // the pushes are read by the next assign; without any, only the
-        // block's own copy moves on
-        if (pushes > 0) {
-            if (!barrier(r)) break;
-        } else {
-            __syncthreads();
-            if (threadIdx.x == 0) h.round = r;
-            __syncthreads();
-        }
+        if (pushes > 0 && !barrier()) break;   // the next assign reads what they wrote
     }
     if (lead) {   // the counters of round r are in place for the core phase
         const int gave_up = *(volatile int*)&st->bar_timeout;
@@ -1486,7 +1581,7 @@ __global__ void d1_core_bits(const Problem<V>* __restrict__ Pp, State* st) {
     for (int i = gw; i < k; i += nw) {
         const int4 e = A.lent[i];
         if (e.y > kCoreWarpList) continue;
-        const int* list = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
+        const int* list = P.hadj + P.g.begin(e.x, e.w);
         for (int b0 = lane; b0 < e.y; b0 += 128) {
             int u[4];
 #pragma unroll
@@ -1499,7 +1594,7 @@ __global__ void d1_core_bits(const Problem<V>* __restrict__ Pp, State* st) {
     for (int i = blockIdx.x; i < k; i += gridDim.x) {
         const int4 e = A.lent[i];
         if (e.y <= kCoreWarpList) continue;   // block-uniform
-        const int* list = P.hadj + P.g.begin(P.g.graph(e.x), e.w);
+        const int* list = P.hadj + P.g.begin(e.x, e.w);
         for (int b = threadIdx.x; b < e.y; b += blockDim.x)
             core_edge(P, i, __ldg(list + b), words);
     }
@@ -1510,7 +1605,7 @@ template <class V>
 __device__ __forceinline__ unsigned forbidden_word(const Problem<V>& P, int4 e, int w) {
     if (w < 2) return __ldcg(reinterpret_cast<const unsigned*>(P.bm0 + e.x) + w);
     if (e.z < 64 || w - 2 > (e.z >> 5)) return 0u;
-    const long long b = P.g.begin(P.g.graph(e.x), e.w);
+    const long long b = P.g.begin(e.x, e.w);
     return __ldcg(P.bmx + P.g.bm(e.x, b) + (w - 2));
 }
 
@@ -1658,7 +1753,7 @@ __device__ __forceinline__ void core_forbid(const Problem<V>& P, const CoreSmem&
     if (gw < 2) {
         atomicOr(reinterpret_cast<unsigned*>(P.bm0 + e.x) + gw, bit);
     } else {
-        const long long b = P.g.begin(P.g.graph(e.x), e.w);
+        const long long b = P.g.begin(e.x, e.w);
         atomicOr(P.bmx + P.g.bm(e.x, b) + (gw - 2), bit);
     }
 }
@@ -1778,7 +1873,6 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
     const bool traced = P.trace_cap > 0 && cta == 0 && warp == 0;
     const unsigned long long t0_ns = st->t0;
     if (traced) {
-        if (lane == 0 && r == 1) P.trace_h[0] = (long long)st->h_first;
         for (int j = lane; j < k; j += 32) {
             const int4 e = A.lent[j];
             sum_s += (unsigned long long)P.g.degree(e.x, e.z);   // per lane, see below
@@ -2057,6 +2151,7 @@ struct Engine {
     cudaGraph_t graph[kGraphs] = {};
     cudaGraphExec_t exec[kGraphs] = {};
     int g_grid = 0, g_block = 0, g_det = 0, g_async = 0, g_dyn = 0;
+    int occ_block = 0, occ_per_sm = 0, occ_det = 0;   // occupancy of the last block size
     int mid_grid = -1;    // blocks of the mid loop (-1: not asked yet)
     bool shares_gpu = false;   // others color on the same GPU: a small mid loop (set once)
     int core_grid = -1;   // CTAs of the core loop's cluster (-1: not asked yet)
@@ -2114,15 +2209,20 @@ struct Engine {
         }
         int per_sm = o.grid_per_sm;
         g->det_grid = dev.num_sms * per_sm;
-        if (per_sm == 0) {
+        if (per_sm == 0 && occ_block == o.block) {
+            per_sm = occ_per_sm;
+            g->det_grid = dev.num_sms * occ_det;
+        } else if (per_sm == 0) {
             int a = 0, b = 0;
             PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, d1_detect<V>, o.block, g->smem));
             if constexpr (V::kSetup)
                 PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, d1_build<V>, o.block, 0));
             else
                 PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, d1_assign<V>, o.block, 0));
-            per_sm = std::max(1, b);
-            g->det_grid = dev.num_sms * std::max(1, a);
+            occ_block = o.block;
+            occ_per_sm = per_sm = std::max(1, b);
+            occ_det = std::max(1, a);
+            g->det_grid = dev.num_sms * occ_det;
         }
         g->grid = dev.num_sms * per_sm;
         if (core_grid < 0) {   // once per engine: does the device take the cluster?
@@ -2140,32 +2240,36 @@ struct Engine {
         }
         g->core_grid = core_grid;
         if (mid_grid < 0) {
-            int per = 0, coop = 0;
-            for (int d = 0; d < (V::kSetup ? 2 : 1); ++d)
-                PGC_CUDA(cudaFuncSetAttribute(mid_func(d), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kMidSmem));
-            PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mid_func(0), kMidThreads,
-                                                                   kMidSmem));
-            if (V::kSetup) {   // both variants run on the same grid
-                int per_dyn = 0;
-                PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_dyn, mid_func(1),
-                                                                       kMidThreads, kMidSmem));
-                per = std::min(per, per_dyn);
+            int fits = 1, coop = 0;   // every variant runs with one block per SM
+            for (int v = 0; v < 4; ++v) {
+                const MidKernel m = mid_kernel(v & 1, v & 2);
+                int per = 0;
+                PGC_CUDA(cudaFuncSetAttribute(m.f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)m.smem()));
+                PGC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, m.f, m.threads,
+                                                                       m.smem()));
+                fits = std::min(fits, per);
             }
             PGC_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev.device));
-            mid_grid = coop && per > 0 ? (shares_gpu ? std::min(kMidShared, dev.num_sms)
-                                                     : dev.num_sms) : 0;
+            mid_grid = coop && fits > 0 ? (shares_gpu ? std::min(kMidShared, dev.num_sms)
+                                                      : dev.num_sms) : 0;
         }
         g->mid_grid = mid_grid;
         return PGC_OK;
     }
 
-    static constexpr size_t kMidSmem = (kMidThreads / 32) * 2 * kIdxSlots * sizeof(int);
-    static void* mid_func(int dyn) {
+    struct MidKernel {
+        void* f;
+        int threads;
+        size_t smem() const { return (size_t)(threads / 32) * 2 * kIdxSlots * sizeof(int); }
+    };
+    // (a server's requests share the GPU: few blocks, each with all its threads)
+    MidKernel mid_kernel(bool dyn, bool small) const {
         if constexpr (V::kSetup) {
-            if (dyn) return (void*)d1_mid<V, true>;
+            if (dyn) return {(void*)d1_mid<V, true, 512>, 512};
         }
-        return (void*)d1_mid<V>;
+        if (small && !shares_gpu) return {(void*)d1_mid<V, false, 512>, 512};
+        return {(void*)d1_mid<V, false, 1024>, 1024};
     }
 
     // launch configuration of the core loop: one cluster
@@ -2209,7 +2313,8 @@ struct Engine {
         return PGC_OK;
     }
 
-    // Setup (optional), round 1 (assign first under PGC_ASYNC) and the WHILE
+    // Setup (optional, with round 1), round 1 when it is not part of the setup
+    // (PGC_ASYNC, round-varying priorities; else its queued pushes) and the WHILE
     // node of the later rounds (both unless small), the mid loop and the core
     // phase.
     pgc_status build_one_graph(const Geometry& g, bool setup, bool small, int async, int dyn,
@@ -2226,7 +2331,9 @@ struct Engine {
         int lo = 0, hi = INT32_MAX;
         State* dS = state.as<State>();
         void* p_args[] = {&dP};
+        int no_cond = 0;
         void* s_args[] = {&dP, &dS};
+        void* n_args[] = {&dP, &dS, &hnd, &no_cond};
         void* b_args[] = {&dP, &lo, &hi};
         void* c_args[] = {&dP, &dS, &hnd, &use_cond};
         cudaMemsetParams ms = {};
@@ -2243,13 +2350,14 @@ struct Engine {
         }
         cudaKernelNodeParams k_det = knode(detect, g, g.smem, c_args);
         k_det.gridDim = dim3(g.det_grid);
-        cudaKernelNodeParams k_push = knode((void*)d1_push<V>, g, 0, s_args);
+        cudaKernelNodeParams k_push = knode((void*)d1_push<V>, g, 0, n_args);
+        cudaKernelNodeParams k_push1 = knode((void*)d1_push<V>, g, 0, c_args);
         cudaKernelNodeParams k_asg = knode((void*)d1_assign<V>, g, 0, c_args);
         if constexpr (V::kSetup) {
             if (setup) {
                 cudaKernelNodeParams k_cls = knode((void*)d1_classify<V>, g, 0, p_args);
                 cudaKernelNodeParams k_build = knode((void*)d1_build<V>, g, 0, b_args);
-                cudaKernelNodeParams k_tier = knode((void*)d1_tier<V>, g, 0, p_args);
+                cudaKernelNodeParams k_tier = knode((void*)d1_tier<V>, g, 0, s_args);
                 PGC_CUDA(cudaGraphAddKernelNode(&n_cls, graph, &n_ms, 1, &k_cls));
                 PGC_CUDA(cudaGraphAddKernelNode(&n_build, graph, &n_cls, 1, &k_build));
                 PGC_CUDA(cudaGraphAddKernelNode(&n_tier, graph, &n_build, 1, &k_tier));
@@ -2265,8 +2373,8 @@ struct Engine {
         };
         if (!small) {
             if (async) PGC_CUDA(after(&n_asg1, graph, k_asg));
-            PGC_CUDA(after(&n_det, graph, k_det));
-            PGC_CUDA(after(&n_push, graph, k_push));
+            if (async || dyn) PGC_CUDA(after(&n_det, graph, k_det));
+            PGC_CUDA(after(&n_push, graph, async || dyn ? k_push : k_push1));
             cudaGraphNodeParams cp = {};
             cp.type = cudaGraphNodeTypeConditional;
             cp.conditional.handle = handle;
@@ -2281,16 +2389,18 @@ struct Engine {
             last = n_loop;
         }
         if (g.mid_grid > 0 && !async) {
-            cudaKernelNodeParams k_mid = knode(mid_func(dyn), g, kMidSmem, s_args);
+            const MidKernel m = mid_kernel(dyn, small);
+            cudaKernelNodeParams k_mid = knode(m.f, g, m.smem(), s_args);
             k_mid.gridDim = dim3(g.mid_grid);
-            k_mid.blockDim = dim3(kMidThreads);
+            k_mid.blockDim = dim3(m.threads);
             cudaGraphNode_t n_mid;
             PGC_CUDA(after(&n_mid, graph, k_mid));
             cudaLaunchAttributeValue coop = {};
             coop.cooperative = 1;
             PGC_CUDA(cudaGraphKernelNodeSetAttribute(n_mid, cudaLaunchAttributeCooperative, &coop));
         }
-        // no-ops unless the mid loop stopped with st->tail set
+        // no-ops unless the mid loop stopped with st->tail set (as a conditional
+        // node, the four launches cost no less when not taken, more when taken)
         if (g.core_grid > 0 && g.mid_grid > 0 && !async && !dyn) {
             cudaKernelNodeParams k_ckeys = knode((void*)d1_core_keys<V>, g, 0, s_args);
             k_ckeys.gridDim = dim3(dev.num_sms);
@@ -2506,7 +2616,7 @@ struct Engine {
                     PGC_CUDA(cudaStreamWaitEvent(stream, up_done[k], 0));
                     d1_build<V><<<g.grid, g.block, 0, stream>>>(dP, cut[k], cut[k + 1]);
                 }
-                d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP);
+                d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP, state.as<State>());
                 PGC_CUDA(cudaGetLastError());
                 PGC_CUDA(cudaGraphLaunch(exec[1], stream));
             }
@@ -2529,29 +2639,35 @@ struct Engine {
                           (d1_classify<V><<<g.grid, g.block, 0, stream>>>(dP)));
                 PGC_TIMED(1, "d1_build",
                           (d1_build<V><<<g.grid, g.block, 0, stream>>>(dP, 0, INT32_MAX)));
-                PGC_TIMED(2, "d1_tier", (d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP)));
+                PGC_TIMED(2, "d1_tier",
+                          (d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP, state.as<State>())));
             } else {   // slot 0 is the caller's
                 if (pgc_status s_ = kt.begin(1, "net_lists")) return s_;
                 if (pgc_status s_ = (*setup)(dP)) return s_;
                 if (pgc_status s_ = kt.end()) return s_;
             }
             for (int round = 1; !small; ++round) {
+                const bool whole = round > 1 || hp->async_mode || hp->prio_mode;
                 if (round > 1 || hp->async_mode)
                     PGC_TIMED(3, "d1_assign",
                               (d1_assign<V><<<g.grid, g.block, 0, stream>>>(dP, dS, none, 0)));
-                if (pgc_status s_ = kt.begin(4, "d1_detect")) return s_;
-                bool dyn_detect = false;
-                if constexpr (V::kSetup) {
-                    if (hp->prio_mode) {
-                        dyn_detect = true;
-                        d1_detect<V, true><<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
+                if (whole) {   // otherwise round 1 was part of the setup
+                    if (pgc_status s_ = kt.begin(4, "d1_detect")) return s_;
+                    bool dyn_detect = false;
+                    if constexpr (V::kSetup) {
+                        if (hp->prio_mode) {
+                            dyn_detect = true;
+                            d1_detect<V, true>
+                                <<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
+                        }
                     }
+                    if (!dyn_detect)
+                        d1_detect<V><<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
+                    PGC_CUDA(cudaGetLastError());
+                    if (pgc_status s_ = kt.end()) return s_;
                 }
-                if (!dyn_detect)
-                    d1_detect<V><<<g.det_grid, g.block, g.smem, stream>>>(dP, dS, none, 0);
-                PGC_CUDA(cudaGetLastError());
-                if (pgc_status s_ = kt.end()) return s_;
-                PGC_TIMED(5, "d1_push", (d1_push<V><<<g.grid, g.block, 0, stream>>>(dP, dS)));
+                PGC_TIMED(5, "d1_push",
+                          (d1_push<V><<<g.grid, g.block, 0, stream>>>(dP, dS, none, 0)));
                 PGC_CUDA(cudaMemcpyAsync(hs, state.ptr, sizeof(State), cudaMemcpyDeviceToHost,
                                          stream));
                 PGC_CUDA(cudaStreamSynchronize(stream));
@@ -2561,9 +2677,10 @@ struct Engine {
             }
             if (hp->mid_w > 0) {   // no-ops once the coloring is done
                 void* args[] = {&dP, &dS};
+                const MidKernel m = mid_kernel(hp->prio_mode != 0, small != 0);
                 if (pgc_status s_ = kt.begin(7, "d1_mid")) return s_;
-                PGC_CUDA(cudaLaunchCooperativeKernel(mid_func(hp->prio_mode != 0), dim3(g.mid_grid),
-                                                     dim3(kMidThreads), args, kMidSmem, stream));
+                PGC_CUDA(cudaLaunchCooperativeKernel(m.f, dim3(g.mid_grid), dim3(m.threads), args,
+                                                     m.smem(), stream));
                 if (pgc_status s_ = kt.end()) return s_;
             }
             if (hp->tail_w > 0) {

@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ 
     const long long gw = (long long)blockIdx.x * wpb + warp, nw = (long long)gridDim.x * wpb;
     const int self = P.self;
     unsigned at = 0u, end = 0u;   // this warp's part of the buffer
-    unsigned long long my_h = 0ull;
+    unsigned long long my_h = 0ull, my_s = 0ull;
     bool full = false;
     for (long long v0 = gw * a.group; v0 < P.n && !full; v0 += nw * a.group) {
         const int count = (int)min((long long)a.group, P.n - v0);
@@ -1098,36 +1098,45 @@ __global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ 
                 }
             }
             if (lane == x) mine = make_int4(v, hi_n, len, (int)at);
+            if (hi_n == 0)   // v commits color 1: forbidden for its neighbors
+                for (int s = lane; s < from_n; s += 32)
+                    if (from[s] != kListEmpty) atomicOr(L.bm0 + from[s], 1ull);
             if (len >= 64)
                 for (int w = lane; w <= len >> 5; w += 32)
                     L.bmx[(long long)v * L.g.bm_words + w] = 0u;
             at += (unsigned)len;
             __syncwarp();
         }
-        const bool have = mine.x >= 0;
+        // round 1 (see d1_tier): vertices without a list commit, the others are
+        // round 2's worklists
+        const bool have = mine.x >= 0, go_on = have && mine.y > 0;
         if (have) {
             a.rows[mine.x] = make_int2(mine.w, mine.z);
-            L.col[mine.x] = -1;
+            L.col[mine.x] = go_on ? -1 : 1;
+            if (!go_on) atomicAnd(L.live + (mine.x >> 5), ~(1u << (mine.x & 31)));
             my_h += (unsigned long long)mine.y;
+            if (go_on && L.trace_cap > 0) my_s += (unsigned long long)(my_k - self);
         }
-        append_warp(have && mine.y <= L.det_s, mine, L.ws[1], &st->ns[1]);
-        append_warp(have && mine.y > L.det_s, mine, L.wm[1], &st->nm[1]);
+        append_warp(go_on && mine.y <= L.det_s, mine, L.ws[0], &st->ns[0]);
+        append_warp(go_on && mine.y > L.det_s, mine, L.wm[0], &st->nm[0]);
     }
     my_h = warp_sum(my_h);
-    if (lane == 0 && my_h) atomicAdd(&st->h_first, my_h);
-    if (full && lane == 0) {
-        st->status = d1::ST_LISTS;
-        st->done = 1;
+    my_s = warp_sum(my_s);
+    if (lane == 0 && my_h) {
+        atomicAdd(&st->h_first, my_h);
+        atomicAdd(&st->h_next, my_h);   // a vertex without a list adds nothing
+        if (my_s) atomicAdd(&st->s_next, my_s);
     }
+    if (full && lane == 0) *(volatile int*)&st->lists_full = 1;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->round = 1;
         st->t0 = global_ns();
-        if (P.n <= L.mid_w) st->mid = 1;
         if (L.trace_cap > 0) {
             L.trace_w[0] = P.n;
             L.trace_s[0] = __ldg(P.r_ptr + P.n);
         }
     }
+    d1::end_round1(L, st);
 }
 
 // ---------------------------------------------------------------------------

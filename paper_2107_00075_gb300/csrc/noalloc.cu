@@ -187,13 +187,15 @@ static pgc_status color_noalloc(int32_t n, const int32_t* row_ptr, const int32_t
     const cudaGraphConditionalHandle none = 0;
     d1_classify<SingleView><<<grid, block, 0, stream>>>(dP);
     d1_build<SingleView><<<grid, block, 0, stream>>>(dP, 0, INT32_MAX);
-    d1_tier<SingleView><<<grid, block, 0, stream>>>(dP);
+    d1_tier<SingleView><<<grid, block, 0, stream>>>(dP, hp.st);   // and round 1
     PGC_CUDA(cudaGetLastError());
     State hs;
     for (int round = 1;; ++round) {
-        if (round > 1) d1_assign<SingleView><<<grid, block, 0, stream>>>(dP, hp.st, none, 0);
-        d1_detect<SingleView><<<grid, block, smem, stream>>>(dP, hp.st, none, 0);
-        d1_push<SingleView><<<grid, block, 0, stream>>>(dP, hp.st);
+        if (round > 1) {
+            d1_assign<SingleView><<<grid, block, 0, stream>>>(dP, hp.st, none, 0);
+            d1_detect<SingleView><<<grid, block, smem, stream>>>(dP, hp.st, none, 0);
+        }
+        d1_push<SingleView><<<grid, block, 0, stream>>>(dP, hp.st, none, 0);
         PGC_CUDA(cudaGetLastError());
         PGC_CUDA(cudaMemcpyAsync(&hs, hp.st, sizeof hs, cudaMemcpyDeviceToHost, stream));
         PGC_CUDA(cudaStreamSynchronize(stream));
