@@ -261,6 +261,62 @@ def d1_algorithmic_bytes(trace_w, trace_s, trace_h, n, nnz, tail_at=None, deg=No
     return out
 
 
+MID_W = 65536    # worklists up to this size: the rounds run in one launch (d1_mid)
+CORE_W = 4096    # ... and, while they shrink slowly, in the core phase (d1_core)
+
+
+def d1_phases(prof):
+    """(mid, core): the 0-based first rounds a profiled (host-loop) coloring
+    ran in d1_mid and in the core phase (the number of rounds when it ran
+    none there), by the engine's rules applied to the trace."""
+    w = [int(x) for x in prof.trace_w]
+    R = len(w)
+    if "d1_mid" not in prof.kernel_ms:
+        return R, R
+    mid = next((i for i in range(1, R) if w[i] <= MID_W), R)
+    core = R
+    if "d1_core" in prof.kernel_ms:
+        core = next((i for i in range(mid + 1, R)
+                     if w[i] <= CORE_W and (w[i - 1] - w[i]) * 8 < w[i]), R)
+    return mid, core
+
+
+def d1_phase_bytes(prof, setup, last_setup, row_mean=None):
+    """Bytes each kernel of a profiled coloring moves: the setup kernels'
+    (setup; round 1 runs in last_setup), then the per-round model of
+    d1_round_bytes split over the launched rounds, d1_mid and the core phase.
+    The core phase's rounds stay in shared memory: it reads, per entry of its
+    worklist's lists, the id, its uncolored word and its rank (12), and per
+    vertex its entry, color and key (28).  row_mean: entries a winner pushes
+    to, when the trace's degrees are not row lengths (conflict lists)."""
+    mid, core = d1_phases(prof)
+    w = np.asarray(prof.trace_w, dtype=np.float64)
+    sw = prof.trace_s if row_mean is None else row_mean * w
+    asg, det, psh = d1_round_bytes(w, sw, prof.trace_h)
+    nb = dict(setup)
+    if len(w):
+        nb[last_setup] += float(det[0] + psh[0])
+    nb["d1_assign"] = float(asg[1:mid].sum())
+    nb["d1_detect"] = float(det[1:mid].sum())
+    nb["d1_push"] = float(psh[1:mid].sum())
+    nb["d1_mid"] = float((asg + det + psh)[mid:core].sum())
+    nb["d1_core"] = float(12 * prof.trace_h[core] + 28 * w[core]) if core < len(w) else 0.0
+    return nb
+
+
+def list_setup_bytes(n, n_nets, memberships, members, h1):
+    """Bytes of the distance-2 setup over conflict lists.  memberships: nets of
+    all vertices, with multiplicity; members: their members; h1: the lists'
+    entries with priority (half of all).
+      net_init:   per vertex offsets 8, key 8, color 4; per net of a vertex its
+                  id 4 and two offsets 8; net flags 4 per net
+      net_lists:  per net of a vertex its id 4 and offsets 8; 4 per member;
+                  per list entry its key 8 and the entry 4; per vertex
+                  offsets 8, key 8, row 8, color 4, worklist entry 16"""
+    return {"net_init": 20.0 * n + 12.0 * memberships + 4.0 * n_nets,
+            "net_lists": 12.0 * memberships + 4.0 * members + 24.0 * h1 + 44.0 * n}
+
+
 def d1_method_bytes(trace_w, trace_s, n, nnz, tail_at=None):
     """Bytes the method's conflict detection must move per round, as the
     method states it (every worklist vertex reads its whole adjacency and
@@ -584,6 +640,8 @@ def bench_batch(pgc, inputs, torch, dev, num_graphs, peak=None, peak_kind="measu
                            colors_per_graph=gc, flags=pgc.PGC_AUTOTUNE, stream=stream)
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     reps = 3
+    for e in (ev0, ev1):   # an event's first record creates it (50 ms once)
+        e.record(stream)
     torch.cuda.synchronize(dev)
     ev0.record(stream)
     for _ in range(reps):
@@ -629,8 +687,7 @@ def bench_batch(pgc, inputs, torch, dev, num_graphs, peak=None, peak_kind="measu
         G = num_graphs
         d = np.diff(b.row_ptr.astype(np.int64))
         deg = np.delete(d, b.vtx_off[1:-1] + np.arange(G - 1))
-        tail_at = d1_split(prof, 4096)
-        nb = d1_algorithmic_bytes(prof.trace_w, prof.trace_s, prof.trace_h, N, E, tail_at, deg)
+        nb = d1_phase_bytes(prof, d1_setup_bytes(N, E, float(prof.trace_h[0]), deg), "d1_tier")
         top = max(prof.kernel_ms, key=prof.kernel_ms.get)
         out["roofline"] = roofline_entry(top, prof.kernel_ms[top], prof.kernel_launches[top],
                                          nb[top], peak, peak_kind, "d1_engine.cuh",
@@ -903,7 +960,7 @@ def bench_net(pgc, inputs, torch, dev, reps=5, warm=2, flags=0, timeout_ms=0, pe
         torch.cuda.synchronize(dev)
         return r, ev0.elapsed_time(ev1) / reps
 
-    def profiled(call, name, n, n_nets, members_total, units, ms):
+    def profiled(call, name, n, n_nets, members_total, units, ms, memberships, members):
         # the per-round trace (for the design bytes) from one host-loop call;
         # the kernel times from a second one without the trace, whose per-net
         # counters detection then skips
@@ -911,14 +968,21 @@ def bench_net(pgc, inputs, torch, dev, reps=5, warm=2, flags=0, timeout_ms=0, pe
         call(pgc.PGC_HOST_LOOP, tprof)
         prof = pgc.Profile(trace_cap=0)
         call(pgc.PGC_HOST_LOOP, prof)
-        nb = net_algorithmic_bytes(tprof.trace_w, tprof.trace_h, tprof.trace_nets,
-                                   tprof.trace_members, n, n_nets, members_total)
+        lists = "net_lists" in prof.kernel_ms
+        if lists:   # rounds over conflict lists
+            h1 = float(tprof.trace_h[0])
+            nb = d1_phase_bytes(tprof, list_setup_bytes(n, n_nets, memberships, members, h1),
+                                "net_lists", row_mean=2.0 * h1 / max(1, n))
+        else:
+            nb = net_algorithmic_bytes(tprof.trace_w, tprof.trace_h, tprof.trace_nets,
+                                       tprof.trace_members, n, n_nets, members_total)
         top = max(prof.kernel_ms, key=prof.kernel_ms.get)
         rf = roofline_entry(top, prof.kernel_ms[top], prof.kernel_launches[top], nb[top], peak,
-                            peak_kind, "net.cu", capture=f"{top} ({name})")
+                            peak_kind, "net.cu" if top.startswith("net_") else "d1_engine.cuh",
+                            capture=f"{top} ({name})")
         if top == "net_detect":
             rf["method_bytes_per_launch"] = nb["method_detect"] / prof.kernel_launches[top]
-        step_bytes = sum(v for k, v in nb.items() if k.startswith("net_"))
+        step_bytes = sum(v for k, v in nb.items() if not k.startswith("method_"))
         return {"roofline": rf, "kernels": kernel_table(prof, nb),
                 "step_bytes": step_bytes,
                 "step_frac": step_bytes / (ms / 1000.0) / 1e9 / peak,
@@ -933,7 +997,9 @@ def bench_net(pgc, inputs, torch, dev, reps=5, warm=2, flags=0, timeout_ms=0, pe
     e = {"workload": "D2, 27-point stencil 128^3", "n": g.n, "nnz": g.nnz, "ms": ms,
          "rounds": r.rounds, "num_colors": r.num_colors, "edges_per_s": (g.nnz / 2) / (ms / 1000)}
     if profile:
-        e.update(profiled(d2, "d2", g.n, g.n, g.nnz + g.n, g.nnz / 2, ms))
+        size = np.diff(g.row_ptr.astype(np.int64)) + 1   # net u: u and its neighbors
+        e.update(profiled(d2, "d2", g.n, g.n, g.nnz + g.n, g.nnz / 2, ms, int(size.sum()),
+                          int((size * size).sum())))
     out["d2_stencil27_128"] = e
     del rp, ci, col
     b = inputs.bipartite(1 << 22, 1 << 20, seed=SEED)
@@ -947,7 +1013,9 @@ def bench_net(pgc, inputs, torch, dev, reps=5, warm=2, flags=0, timeout_ms=0, pe
          "rows": b.n_rows, "cols": b.n_cols, "nnz": b.nnz, "ms": ms, "rounds": r.rounds,
          "num_colors": r.num_colors, "edges_per_s": b.nnz / (ms / 1000)}
     if profile:
-        e.update(profiled(pd2, "pd2", b.n_cols, b.n_rows, b.nnz, b.nnz, ms))
+        size = np.diff(b.row_ptr.astype(np.int64))
+        e.update(profiled(pd2, "pd2", b.n_cols, b.n_rows, b.nnz, b.nnz, ms, b.nnz,
+                          int((size * size).sum())))
     out["pd2_4Mx1M"] = e
     return out
 
@@ -1153,11 +1221,10 @@ def main():
                        "trace_s": prof.trace_s.tolist(), "trace_h": prof.trace_h.tolist()},
                       open(args.dump_profile, "w"))
         trace_w = prof.trace_w
-        tail_w = 4096 if args.tail_vertices == 0 else args.tail_vertices
-        tail_at = d1_split(prof, tail_w)
+        mid_at, _ = d1_phases(prof)
         launches_per_step = d1_kernel_launches(prof)
-        nbytes = d1_algorithmic_bytes(prof.trace_w, prof.trace_s, prof.trace_h, n, nnz,
-                                      tail_at, deg)
+        nbytes = d1_phase_bytes(prof, d1_setup_bytes(n, nnz, float(prof.trace_h[0]), deg),
+                                "d1_tier")
         kernels = kernel_table(prof, nbytes)
         top = max(prof.kernel_ms, key=prof.kernel_ms.get)
         launches = prof.kernel_launches[top]
@@ -1166,7 +1233,7 @@ def main():
         # the method's own per-round adjacency scan, for context: this design
         # does not move those bytes (it scans priority lists and stops early)
         if top == "d1_detect":
-            tot, _ = d1_method_bytes(prof.trace_w, prof.trace_s, n, nnz, tail_at)
+            tot, _ = d1_method_bytes(prof.trace_w, prof.trace_s, n, nnz, mid_at)
             roofline["method_bytes_per_launch"] = tot / launches
         step_bytes = float(sum(nbytes.values()))
         roofline["step_bytes"] = step_bytes
@@ -1176,8 +1243,8 @@ def main():
     small = net = batch = serve = None
     if rank == 0 and not args.no_small:
         sg, small, sprof = bench_small_d1(pgc, inputs, torch, dev)
-        sb = d1_algorithmic_bytes(sprof.trace_w, sprof.trace_s, sprof.trace_h, sg.n, sg.nnz,
-                                  d1_split(sprof, 4096), np.diff(sg.row_ptr))
+        sb = d1_phase_bytes(sprof, d1_setup_bytes(sg.n, sg.nnz, float(sprof.trace_h[0]),
+                                                  np.diff(sg.row_ptr)), "d1_tier")
         stop = max(sprof.kernel_ms, key=sprof.kernel_ms.get)
         small["roofline"] = roofline_entry(stop, sprof.kernel_ms[stop],
                                            sprof.kernel_launches[stop], sb[stop], peak,

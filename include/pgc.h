@@ -107,7 +107,8 @@ typedef enum {
 typedef struct {
     /* per-round trace, entry r describes round r+1's worklist W_{r+1}:
        w[r] = |W_{r+1}|, s[r] = sum of deg(v), h[r] = sum of the lengths of
-       the detection lists (D1: neighbors with higher priority) */
+       the detection lists (neighbors, or for D2/PD2 vertices of a common net,
+       with higher priority; D2/PD2 in net rounds: the vertices' nets) */
     int64_t *trace_w;          /* host array of trace_cap entries, or NULL */
     int64_t *trace_s;          /* host array of trace_cap entries, or NULL */
     int64_t *trace_h;          /* host array of trace_cap entries, or NULL */
@@ -127,7 +128,8 @@ typedef struct {
     int32_t num_launches;
     /* D2/PD2 only, nullable host arrays of trace_cap entries: entry r-1
        describes round r's detection -- the nets it visited (every net, or
-       those with a member on the worklist) and their total member count */
+       those with a member on the worklist) and their total member count; all
+       zero when the rounds ran over conflict lists, which visit no net */
     int64_t *trace_nets;
     int64_t *trace_members;
 } pgc_profile;
@@ -136,17 +138,17 @@ typedef struct {
     uint32_t flags;            /* PGC_* flags above */
     int32_t max_rounds;        /* 0 => n + 1 (an upper bound: each round commits
                                   the worklist vertex with the largest key) */
-    int32_t mid_degree;        /* 0 => 64: a vertex whose per-round scan list
-                                  (D1: neighbors with higher priority) is longer
-                                  gets a warp instead of a thread */
-    int32_t hub_degree;        /* 0 => 16384: longer lists get a thread block */
+    int32_t mid_degree;        /* D1; 0 => 64: vertices whose per-round scan list
+                                  (neighbors with higher priority) is longer are
+                                  kept, and searched by warps, apart */
+    int32_t hub_degree;        /* D1; 0 => 16384: longer lists get a thread block */
     int32_t block;             /* 0 => default threads per block (128..1024) */
     int32_t grid_per_sm;       /* 0 => occupancy-derived blocks per SM */
     int32_t timeout_ms;        /* 0 => 60000: device loop gives up after this */
     int32_t tail_vertices;     /* D1: once the worklist has at most this many
-                                  vertices, the remaining rounds run on the
-                                  subgraph the worklist induces, in one
-                                  cooperative launch with grid barriers;
+                                  vertices (4096 at most) and shrinks slowly,
+                                  the remaining rounds run on the subgraph it
+                                  induces, in one thread-block cluster;
                                   0 => 4096, < 0 => never */
     pgc_profile *profile;      /* nullable */
 } pgc_opts;
