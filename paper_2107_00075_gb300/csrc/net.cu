@@ -889,13 +889,13 @@ __global__ void net_commit(const Problem* __restrict__ Pp, cudaGraphConditionalH
 // one counter in chunks, in any order.
 //
 // Bound by issue (about 2,500 warp instructions per vertex of the 27-point
-// mesh 128^3, 6.0 ms for its 2.1M vertices; PD2 4M x 1M 4.6 ms).  A hash that
+// mesh 128^3, 6.3 ms for its 2.1M vertices; PD2 4M x 1M 4.2 ms).  A hash that
 // kept blocks of 32 ids together put whole runs of a mesh on top of each
 // other (39 ms); reading the set out slot by slot took 10 ms.
 //
 // With lists the whole coloring of the mesh takes 13.7 ms (22.5 in net
-// rounds), of PD2 4M x 1M 12.0 ms (21.9), of PD2 40K x 10K 1.1 ms (3.3), of a
-// 7-point mesh of 51,615 vertices 0.39 ms (0.75).
+// rounds), of PD2 4M x 1M 11.5 ms (21.9), of PD2 40K x 10K 0.94 ms (3.4), of a
+// 7-point mesh of 51,615 vertices 0.34 ms (0.76).
 // ---------------------------------------------------------------------------
 constexpr int kListMinLog = 6, kListMaxLog = 11;          // log2 of a warp's hash set
 constexpr int kListMid = 64;                              // lists up to this length: S tier

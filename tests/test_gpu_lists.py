@@ -88,3 +88,15 @@ def test_random_patterns_and_both_sides(n_cols):
 @pytest.mark.parametrize("points", [7, 27])
 def test_meshes(shape, points):
     check_d2(gen.stencil3d(*shape, points=points), seed=sum(shape))
+
+
+def test_repeats_after_distinct_members():
+    """A warp that saw few repeats among members skips the hash set; the columns
+    after such a one share five equal rows with their neighbors here, so their
+    lists then hold repeats, which must change nothing."""
+    n = 24000
+    b = gen.bipartite(3 * n // 4, n // 4, seed=8)
+    rows = [(4 * b.col_idx[b.row_ptr[i]:b.row_ptr[i + 1]]).tolist() for i in range(b.n_rows)]
+    for q in range(0, n, 4):
+        rows += [[q + 1, q + 2, q + 3]] * 5
+    check_pd2(_graphs.bipartite_from_rows(rows, n), seed=3)
