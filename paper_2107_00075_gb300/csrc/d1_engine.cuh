@@ -164,9 +164,14 @@ constexpr int kBuildS = 32;     // setup: degree up to this: one thread
 constexpr int kBuildM = 512;    // setup: degree up to this: one warp
 constexpr int kBuildItem = 512; // setup: adjacency items of this length
 constexpr int kPushItem = 128;  // push: adjacency items of this length
-// round-varying priorities: longer lists take a block (R-MAT 18, dynamic degree:
-// 14.0 ms with one warp up to 16,384 entries, 5.2 ms)
-constexpr int kVaryingHub = 1024;
+// round-varying priorities: longer lists take a block.  A small graph has few
+// of them and a warp on one is what a round waits for; a large one has enough
+// long lists to fill the grid, and blocks on the shorter of them wait at their
+// barriers.  Dynamic degree, edge factor 16, with blocks from 1024 / 2048 / 4096
+// entries up: R-MAT 18 4.2 / 5.3 / 5.3 ms, R-MAT 20 12.7 / 11.1 / 16.0 ms, R-MAT 21
+// 22.0 / 19.0 / 18.9 ms, R-MAT 22 39.3 / 38.6 / 34.0 ms, R-MAT 24 191 / 190 / 152 ms
+// (from 16,384 up: R-MAT 22 55 ms, R-MAT 24 155 ms)
+inline int varying_hub(int n) { return std::clamp(n >> 9, 1024, 4096); }
 // winners up to this degree push inline: 32 / 128 / 512 take 73.7 / 58.5 / 58.5 ms
 // for the 4096-graph batch and 3.68 / 3.66 / 4.05 ms for R-MAT 20
 constexpr int kInlinePush = 128;
@@ -2557,7 +2562,7 @@ struct Engine {
         hp->det_s = o.mid_degree;
         // lists that hold whole rows: hubs' lists are long, and a block reads 1024
         // entries per step where a warp reads 128
-        hp->det_m = pflags ? std::max(o.mid_degree, std::min(o.hub_degree, kVaryingHub))
+        hp->det_m = pflags ? std::max(o.mid_degree, std::min(o.hub_degree, varying_hub((int)n)))
                            : o.hub_degree;
         hp->mid_w = hp->async_mode || g.mid_grid == 0 ? 0 : shares_gpu ? kMidSharedMax : kMidMax;
         hp->tail_w = hp->mid_w == 0 || pflags || g.core_grid == 0

@@ -50,3 +50,24 @@ def _core_with_hub(leaves, clique):
 @pytest.mark.parametrize("leaves", [3000, 5000, 20000])
 def test_long_rows(leaves):
     check(_core_with_hub(leaves, 70), seed=leaves)
+
+
+@pytest.mark.parametrize("n,hub", [(1 << 17, 1024), (1 << 20, 2048), (1 << 21, 4096)])
+@pytest.mark.parametrize("prio", ["DYNAMIC", "SATURATION"])
+def test_varying_hubs(n, hub, prio):
+    """Round-varying priorities: the length from which a list takes a block grows
+    with n; hubs one short of it, at it and past it, joined into a clique."""
+    import torch
+    import paper_2107_00075_gb300 as pgc
+    degrees = [hub - 1, hub, hub + 1, 2 * hub]
+    k, edges, at = len(degrees), [], len(degrees)
+    for i, d in enumerate(degrees):
+        edges += [(i, j) for j in range(i + 1, k)]
+        edges += [(i, at + j) for j in range(d - k + 1)]
+        at += d - k + 1
+    g = gen.from_edge_list(n, edges)
+    r = pgc.pgc_color_d1(torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col_idx).cuda(),
+                         seed=5, flags=getattr(pgc, "PGC_PRIORITY_" + prio))
+    want = oracle.color_d1_priority(g.row_ptr, g.col_idx, getattr(oracle, "PRIO_" + prio), seed=5)
+    assert (r.rounds, r.num_colors) == (want.rounds, want.num_colors)
+    assert np.array_equal(r.colors.cpu().numpy(), want.colors)
