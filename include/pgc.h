@@ -362,23 +362,28 @@ const char *pgc_version(void);
 
 /*
  * Test hooks: fault injection for the failure-path tests (no production use;
- * the paper has no counterpart).  Both act process-wide on later calls.
+ * the paper has no counterpart).  They act process-wide on later calls.
  *
  * pgc_test_fail_alloc(after): the device allocation the library attempts
  *   after `after` further successful ones fails as if the device were out of
  *   memory, once; the call that meets it returns PGC_ERR_OOM having freed
  *   the scratch of that engine.  after < 0 disarms.
- * pgc_test_core_barrier(polls, slow_block, slow_us): the grid barrier of the
- *   D1 core loop gives up after `polls` polls (0: the default, about one
- *   second), and block `slow_block` of the core loop (-1: none) reaches its
- *   first barrier `slow_us` microseconds late (at most 2 s, else
- *   PGC_ERR_INVALID_ARG).  With a late block and a short poll limit the
- *   waiting blocks give up, and the coloring returns PGC_ERR_TIMEOUT ("a
- *   grid barrier of the core loop timed out") with the context intact; every
- *   wait stays bounded.
+ * pgc_test_core_barrier(polls, slow_block, slow_us): the blocks of the core
+ *   loop (the last rounds, one thread-block cluster) meet before its first
+ *   round; the meeting gives up after `polls` polls (0: the default, about one
+ *   second), and block `slow_block` (-1: none) reaches it `slow_us`
+ *   microseconds late (at most 2 s, else PGC_ERR_INVALID_ARG).  With a late
+ *   block and a short poll limit the waiting blocks give up, and the coloring
+ *   returns PGC_ERR_TIMEOUT ("a grid barrier of the core loop timed out") with
+ *   the context intact.
+ * pgc_test_mid_barrier(polls, slow_block, slow_us, at): the same for the loop
+ *   that runs the rounds of small worklists in one launch; its block
+ *   `slow_block` is late at its at-th grid barrier (1: the first), and the
+ *   message is "a grid barrier of the mid loop timed out".
  */
 pgc_status pgc_test_fail_alloc(int32_t after);
 pgc_status pgc_test_core_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us);
+pgc_status pgc_test_mid_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us, int32_t at);
 
 #ifdef __cplusplus
 }

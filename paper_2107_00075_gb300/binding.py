@@ -144,6 +144,8 @@ def lib():
         L.pgc_test_fail_alloc.restype = ctypes.c_int
         L.pgc_test_core_barrier.argtypes = [ctypes.c_uint32, i32, ctypes.c_uint32]
         L.pgc_test_core_barrier.restype = ctypes.c_int
+        L.pgc_test_mid_barrier.argtypes = [ctypes.c_uint32, i32, ctypes.c_uint32, i32]
+        L.pgc_test_mid_barrier.restype = ctypes.c_int
         _declared = True
     return L
 
@@ -457,6 +459,12 @@ def pgc_test_core_barrier(polls: int = 0, slow_block: int = -1, slow_us: int = 0
     """Test hook: poll limit of the core loop's grid barrier (0: default) and
     a late core-loop block (-1: none); see pgc.h."""
     _check(lib().pgc_test_core_barrier(polls, slow_block, slow_us))
+
+
+def pgc_test_mid_barrier(polls: int = 0, slow_block: int = -1, slow_us: int = 0, at: int = 1):
+    """Test hook: the same for the mid loop's grid barriers; the block is late
+    at its at-th one (see pgc.h)."""
+    _check(lib().pgc_test_mid_barrier(polls, slow_block, slow_us, at))
 
 
 def pgc_release():

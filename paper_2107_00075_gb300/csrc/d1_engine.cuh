@@ -46,7 +46,10 @@
 // mid_w vertices the rounds run in one cooperative launch with grid barriers
 // (the mid loop), and the last ones of a dense core on the subgraph the
 // worklist induces, in one thread-block cluster (the core phase).  Their
-// barriers are the only waits in the engine; they are bounded.
+// waits are the only ones in the engine: the mid loop's barriers and the
+// cluster's first meeting poll with a limit; the core's rounds use the hardware
+// cluster barrier, which has none, between CTAs that have all met and do
+// finite work.
 //
 // Batches: graph g owns global vertices [vtx_off[g], vtx_off[g+1]); ids,
 // the priority hash and degrees are graph-local, so every graph is colored
@@ -178,7 +181,8 @@ constexpr int kInlinePush = 128;
 
 enum : int {
     ST_OK = 0, ST_NO_PROGRESS = 1, ST_MAX_ROUNDS = 2, ST_TIMEOUT = 3, ST_BARRIER = 4,
-    ST_LISTS = 5   // ListView: the lists did not fit their buffer
+    ST_LISTS = 5,  // ListView: the lists did not fit their buffer
+    ST_MID_BARRIER = 6   // (ST_BARRIER: the core phase's meeting)
 };
 
 // What every block of a round's kernel reads, in one place: a block reads it
@@ -253,9 +257,13 @@ struct Problem {
     int det_m;
     int mid_w;         // hand over to the mid loop once the worklist is this small (0: never)
     int tail_w;        // core phase for worklists up to this size (0: never)
-    unsigned bar_polls;   // core loop: barrier polls before giving up
-    int slow_block;       // test hook: this core-loop CTA starts late (-1: none)
-    unsigned slow_ns;     // ... by this much
+    // a wait's limit, and the test hook's late block
+    struct Wait {
+        unsigned polls;     // polls before giving up
+        int slow_block;     // this block is late (-1: none)
+        unsigned slow_ns;   // ... by this much
+        int slow_at;        // ... at its slow_at-th barrier (mid loop)
+    } mid_wait, core_wait;  // the mid loop's barriers, the core phase's meeting
 };
 
 // A block's copy of the problem and of the round's counters.  Kernels take
@@ -1279,6 +1287,12 @@ __global__ void d1_push(const Problem<V>* __restrict__ Pp, State* st,
 // ---------------------------------------------------------------------------
 // mid loop: the rounds of a worklist that does not fill the GPU
 // ---------------------------------------------------------------------------
+// Test hook: the calling thread waits ns nanoseconds (the host sets at most 2 s).
+__device__ __forceinline__ void be_late(unsigned ns) {
+    const unsigned long long t_end = global_ns() + ns;
+    while (global_ns() < t_end) __nanosleep(1000);
+}
+
 // Grid-wide barrier for a cooperative launch (all blocks co-resident), then
 // the block's copy of the counters.  Arrivals only count up and everyone polls
 // the count itself, so nobody waits for an atomic's answer or for a second
@@ -1355,13 +1369,13 @@ __global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp
     Hot& h = ctx.h;
     if (h.done || !h.mid) return;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    if ((int)blockIdx.x == P.slow_block && threadIdx.x == 0) {
-        // test hook: this block reaches its first barrier late (bounded)
-        const unsigned long long t_end = global_ns() + P.slow_ns;
-        while (global_ns() < t_end) __nanosleep(1000);
-    }
     unsigned phase = 0u;
-    auto barrier = [&] { return grid_barrier(st, h, phase, P.bar_polls); };
+    auto barrier = [&] {
+        if ((int)blockIdx.x == P.mid_wait.slow_block && (int)phase + 1 == P.mid_wait.slow_at &&
+            threadIdx.x == 0)
+            be_late(P.mid_wait.slow_ns);
+        return grid_barrier(st, h, phase, P.mid_wait.polls);
+    };
     int r = h.round, cur = h.count(r & 1), status = ST_OK, done = 0, tail = 0;
     const unsigned long long t0 = lead ? st->t0 : 0ull;
     bool ok = true;
@@ -1407,7 +1421,7 @@ __global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp
     if (lead) {   // the counters of round r are in place for the core phase
         const int gave_up = *(volatile int*)&st->bar_timeout;
         st->round = r;
-        st->status = gave_up ? ST_BARRIER : status;
+        st->status = gave_up ? ST_MID_BARRIER : status;
         st->done = gave_up || done || status != ST_OK;
         st->tail = tail;
         st->mid = 0;
@@ -1886,17 +1900,13 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
     }
     __syncthreads();
     cluster_sync();   // every CTA's shared memory is ready for its peers
-    if (cta == P.slow_block && tid == 0) {
-        // test hook: this CTA reaches the meeting late (bounded)
-        const unsigned long long t_end = global_ns() + P.slow_ns;
-        while (global_ns() < t_end) __nanosleep(1000);
-    }
+    if (cta == P.core_wait.slow_block && tid == 0) be_late(P.core_wait.slow_ns);
     // what a round needs of the problem, kept in registers: after a cluster
     // barrier a global load is an L2 round trip
     const int max_rounds = P.max_rounds, trace_cap = P.trace_cap;
     const unsigned long long timeout_ns = P.timeout_ns;
     int cur = k, status = ST_OK;
-    core_meet(X, C, P.bar_polls);
+    core_meet(X, C, P.core_wait.polls);
     cluster_sync();
     // a CTA may have given up after this one met everyone: all decide by the
     // flag, which every CTA holds by now
@@ -2569,9 +2579,8 @@ struct Engine {
                          ? 0 : std::min(o.tail_vertices, kCoreMax);
         const int small = n <= hp->mid_w ? 2 : 0;
         const TestHooks th = test_hooks();
-        hp->bar_polls = th.barrier_polls;
-        hp->slow_block = th.slow_block;
-        hp->slow_ns = th.slow_us * 1000u;
+        hp->mid_wait = {th.mid.polls, th.mid.slow_block, th.mid.slow_us * 1000u, th.mid.at};
+        hp->core_wait = {th.core.polls, th.core.slow_block, th.core.slow_us * 1000u, th.core.at};
         PGC_CUDA(cudaMemcpyAsync(problem.ptr, hp, sizeof(Problem<V>), cudaMemcpyHostToDevice,
                                  stream));
         Problem<V>* dP = problem.as<Problem<V>>();
@@ -2735,6 +2744,8 @@ struct Engine {
             case ST_TIMEOUT: return fail(PGC_ERR_TIMEOUT, "device round loop exceeded timeout_ms");
             case ST_BARRIER:
                 return fail(PGC_ERR_TIMEOUT, "a grid barrier of the core loop timed out");
+            case ST_MID_BARRIER:
+                return fail(PGC_ERR_TIMEOUT, "a grid barrier of the mid loop timed out");
             default: return fail(PGC_ERR_CUDA, "unexpected device status");
         }
     }

@@ -171,8 +171,6 @@ static pgc_status color_noalloc(int32_t n, const int32_t* row_ptr, const int32_t
     hp.det_s = defaults.mid_degree;
     hp.det_m = defaults.hub_degree;
     hp.tail_w = 0;
-    hp.bar_polls = 1u << 22;
-    hp.slow_block = -1;
     auto* dP = reinterpret_cast<Problem<SingleView>*>(base + L::problem);
     DrainOnExit drain{stream};
     drain.armed = true;

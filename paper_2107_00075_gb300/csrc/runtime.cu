@@ -177,7 +177,16 @@ std::vector<std::function<void()>>& release_hooks() {
     return h;
 }
 
+static void set_wait(TestHooks::Wait& w, unsigned polls, int slow_block, unsigned slow_us, int at) {
+    w.polls = polls == 0 ? TestHooks::Wait().polls : polls;
+    w.slow_block = slow_block;
+    w.slow_us = slow_block < 0 ? 0u : slow_us;
+    w.at = at;
+}
+
 }  // namespace pgc
+
+using pgc::set_wait;
 
 extern "C" {
 
@@ -219,9 +228,16 @@ pgc_status pgc_test_core_barrier(uint32_t polls, int32_t slow_block, uint32_t sl
     if (slow_us > 2000000u)
         return pgc::fail(PGC_ERR_INVALID_ARG, "pgc_test_core_barrier: slow_us above 2 s");
     std::lock_guard<std::mutex> lk(pgc::g_hooks_mu);
-    pgc::g_hooks.barrier_polls = polls == 0 ? (1u << 22) : polls;
-    pgc::g_hooks.slow_block = slow_block;
-    pgc::g_hooks.slow_us = slow_block < 0 ? 0u : slow_us;
+    set_wait(pgc::g_hooks.core, polls, slow_block, slow_us, 1);
+    return PGC_OK;
+}
+
+pgc_status pgc_test_mid_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us, int32_t at) {
+    if (slow_us > 2000000u)
+        return pgc::fail(PGC_ERR_INVALID_ARG, "pgc_test_mid_barrier: slow_us above 2 s");
+    if (at < 1) return pgc::fail(PGC_ERR_INVALID_ARG, "pgc_test_mid_barrier: at < 1");
+    std::lock_guard<std::mutex> lk(pgc::g_hooks_mu);
+    set_wait(pgc::g_hooks.mid, polls, slow_block, slow_us, at);
     return PGC_OK;
 }
 

@@ -45,10 +45,14 @@ bool is_host_pointer(const void* p);
 
 // Fault-injection settings of the test hooks (pgc_test_* in pgc.h).
 struct TestHooks {
-    int fail_alloc_after = -1;          // allocations left before one fails (-1: off)
-    unsigned barrier_polls = 1u << 22;  // core-loop grid barrier: polls before giving up
-    int slow_block = -1;                // core loop: this block arrives late (-1: none)
-    unsigned slow_us = 0;               // ... by this many microseconds
+    int fail_alloc_after = -1;      // allocations left before one fails (-1: off)
+    // a wait among blocks: its limit, and one block that reaches it late
+    struct Wait {
+        unsigned polls = 1u << 22;  // polls before giving up (about a second)
+        int slow_block = -1;        // this block is late (-1: none)
+        unsigned slow_us = 0;       // ... by this many microseconds
+        int at = 1;                 // ... at its at-th barrier (mid loop)
+    } core, mid;                    // the core phase's meeting, the mid loop's barriers
 };
 TestHooks test_hooks();                 // a snapshot
 bool test_take_alloc_failure();         // true if this allocation must fail
