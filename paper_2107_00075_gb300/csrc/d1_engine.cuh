@@ -1844,8 +1844,17 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
     State* st = P.st;
     // uniform over the cluster: nothing has been shared yet
     if (*(volatile int*)&st->done || !*(volatile int*)&st->tail) return;
-    constexpr int C = kCoreCluster;
     const int cta = blockIdx.x;
+    // A block of the mid loop may have given up at its last barrier just as the
+    // others passed it, too late for their report: its pushes are missing.
+    if (*(volatile int*)&st->bar_timeout) {
+        if (cta == 0 && threadIdx.x == 0) {
+            st->status = ST_MID_BARRIER;
+            st->done = 1;
+        }
+        return;
+    }
+    constexpr int C = kCoreCluster;
     const int k = st->core_k, words = core_words(k), words4 = (k + 127) >> 7;
     const int rtl = core_rt_log(k), Rt = 1 << rtl;
     const CoreArrays A = core_arrays(P, st->core_par, k);
