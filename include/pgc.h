@@ -380,10 +380,16 @@ const char *pgc_version(void);
  *   that runs the rounds of small worklists in one launch; its block
  *   `slow_block` is late at its at-th grid barrier (1: the first), and the
  *   message is "a grid barrier of the mid loop timed out".
+ * pgc_test_list_room(limit, buffer): distance-2 and partial distance-2 colorings
+ *   over conflict lists: the lists may take at most `limit` entries (0: the
+ *   default, 2^29), which decides whether they are built, and their buffer gets
+ *   at most `buffer` (0: no limit), so that a build runs out of room.  The
+ *   problem is then colored in net rounds, with the same result.
  */
 pgc_status pgc_test_fail_alloc(int32_t after);
 pgc_status pgc_test_core_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us);
 pgc_status pgc_test_mid_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us, int32_t at);
+pgc_status pgc_test_list_room(uint32_t limit, uint32_t buffer);
 
 #ifdef __cplusplus
 }

@@ -10,5 +10,5 @@ from .binding import (  # noqa: F401
     PgcError, PgcServer, Profile, RequestInfo, pgc_color_d1, pgc_color_d1_batch,
     pgc_color_d1_noalloc, pgc_color_d2, pgc_color_pd2, pgc_color_pd2_bipartite, pgc_release,
     pgc_test_core_barrier,
-    pgc_test_fail_alloc, pgc_test_mid_barrier, pgc_version,
+    pgc_test_fail_alloc, pgc_test_list_room, pgc_test_mid_barrier, pgc_version,
 )

@@ -146,6 +146,8 @@ def lib():
         L.pgc_test_core_barrier.restype = ctypes.c_int
         L.pgc_test_mid_barrier.argtypes = [ctypes.c_uint32, i32, ctypes.c_uint32, i32]
         L.pgc_test_mid_barrier.restype = ctypes.c_int
+        L.pgc_test_list_room.argtypes = [ctypes.c_uint32, ctypes.c_uint32]
+        L.pgc_test_list_room.restype = ctypes.c_int
         _declared = True
     return L
 
@@ -465,6 +467,12 @@ def pgc_test_mid_barrier(polls: int = 0, slow_block: int = -1, slow_us: int = 0,
     """Test hook: the same for the mid loop's grid barriers; the block is late
     at its at-th one (see pgc.h)."""
     _check(lib().pgc_test_mid_barrier(polls, slow_block, slow_us, at))
+
+
+def pgc_test_list_room(limit: int = 0, buffer: int = 0):
+    """Test hook: entries the conflict lists of D2/PD2 may take, and those their
+    buffer gets at most (0: the defaults); see pgc.h."""
+    _check(lib().pgc_test_list_room(limit, buffer))
 
 
 def pgc_release():

@@ -70,6 +70,7 @@ struct State {
     int members;      // max over v of sum over its nets of |net|
     unsigned long long pairs;          // sum over v of sum over its nets of (|net| - 1)
     unsigned long long list_next;      // conflict lists: entries handed out
+    unsigned long long sample_pairs, sample_entries;   // net_list_sample's sums
 };
 
 struct Problem {
@@ -900,7 +901,8 @@ __global__ void net_commit(const Problem* __restrict__ Pp, cudaGraphConditionalH
 constexpr int kListMinLog = 6, kListMaxLog = 11;          // log2 of a warp's hash set
 constexpr int kListMid = 64;                              // lists up to this length: S tier
 constexpr unsigned kListEmpty = 0xffffffffu;              // no id: ids are below 2^31 - 1
-constexpr unsigned long long kListMaxEntries = 1ull << 29;   // 2 GB of lists
+constexpr unsigned long long kListMaxEntries = 1ull << 29;   // 2 GB of lists: what a coloring
+                                                             // keeps on the device for the next
 
 struct ListArgs {
     int2* rows;          // {first entry, length} per vertex
@@ -928,6 +930,49 @@ __device__ __forceinline__ bool list_insert(unsigned* set, int log, int u) {
         const unsigned old = atomicCAS(set + h, kListEmpty, (unsigned)u);
         if (old == kListEmpty) return true;
         if (old == (unsigned)u) return false;
+    }
+}
+
+// How many entries the lists take, per pair (a member of a net of a vertex other
+// than the vertex): a mesh lists a neighbor many times (124 entries of 676 pairs
+// on the 27-point mesh), a random pattern hardly ever twice.  One vertex out of
+// each of `count` equal parts of the ids, at a hashed place, one warp each.
+// Asked for before a build that the number of pairs alone would not admit
+// (d2_mesh27_128: about 0.05 of 14 ms).
+constexpr int kListSample = 4096;
+__global__ void __launch_bounds__(256) net_list_sample(const Problem* __restrict__ Pp, int log,
+                                                       int count, int may_keep) {
+    extern __shared__ uint4 list_sm[];
+    const Problem& P = *Pp;
+    const int lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    unsigned* const set = reinterpret_cast<unsigned*>(list_sm) + (warp << log);
+    unsigned long long pairs = 0ull, entries = 0ull;
+    for (int s = blockIdx.x * wpb + warp; s < count; s += gridDim.x * wpb) {
+        const long long lo = (long long)P.n * s / count, hi = (long long)P.n * (s + 1) / count;
+        const int v = (int)(lo + (long long)(prio_hash(P.seed, (uint32_t)s) %
+                                             (unsigned long long)(hi - lo)));
+        for (int i = lane; i < (1 << log); i += 32) set[i] = kListEmpty;
+        __syncwarp();
+        const int beg = __ldg(P.r_ptr + v), k = __ldg(P.r_ptr + v + 1) - beg + P.self;
+        int members = 0, found = 0;
+        for (int j = 0; j < k; ++j) {
+            const int q = vertex_net(P, v, beg, j), size = net_size(P, q);
+            members += size;
+            for (int m = 0; m < size; m += 32) {
+                const int u = m + lane < size ? net_member(P, q, m + lane) : -1;
+                const bool is_new = list_insert(set, log, u == v ? -1 : u);
+                found += __popc(__ballot_sync(kFullMask, is_new));
+            }
+        }
+        // (net_lists keeps the repeats where they are few)
+        const bool keeps = may_keep && k <= 32 && 8 * (members - k - found) <= members;
+        pairs += (unsigned long long)(members - k);
+        entries += (unsigned long long)(keeps ? max(members - k, found) : found);
+        __syncwarp();
+    }
+    if (lane == 0 && pairs) {
+        atomicAdd(&P.st->sample_pairs, pairs);
+        atomicAdd(&P.st->sample_entries, entries);
     }
 }
 
@@ -1343,23 +1388,27 @@ static pgc_status run(Context& cx, const Input& in, int nnz, uint64_t seed, cons
 // The coloring as a distance-1 coloring of the conflict graph, once net_init
 // has run and hs holds its sums.  *taken is false when the problem is left to
 // the net rounds: a vertex with too many members for a warp's set, lists that
-// would not fit kListMaxEntries, or no device memory for them.
+// would not fit kListMaxEntries, or no device memory for them.  The net rounds
+// then find the memory that the lists held free again.
 static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& hs, uint64_t seed,
                             const Opts& o, cudaStream_t stream, int* rounds, int* num_colors,
                             bool* taken) {
     using E = d1::Engine<d1::ListView>;
     *taken = false;
     const int n = in.n;
-    if (hs.members >= 1 << kListMaxLog || hs.pairs > 8 * kListMaxEntries) return PGC_OK;
+    if (hs.members >= 1 << kListMaxLog) return PGC_OK;
     E* eng = d1::engine_for<d1::ListView>(cx.dev.device);
     std::lock_guard<std::mutex> lk(eng->mu);
     eng->dev = cx.dev;
+    const TestHooks th = test_hooks();
+    const unsigned long long limit = th.list_limit ? th.list_limit : kListMaxEntries;
 
     ListArgs a = {};
     a.log = kListMinLog;
     while (1 << a.log <= hs.members) ++a.log;
     a.members = hs.members;
     const int block = 256, wpb = block / 32;
+    const Problem* dP = cx.problem.as<Problem>();
     const size_t smem = (size_t)wpb * list_warp_ints(a.log) * 4;
     if (smem > 48 * 1024)
         PGC_CUDA(cudaFuncSetAttribute(net_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1373,9 +1422,40 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
     // the next row does not fit: less than a row in 8, and a part per warp.
     a.group = (int)std::max<long long>(1, std::min<long long>(32, n / warps));
     a.chunk = n >= 8 * warps ? 8u * (unsigned)hs.members : 0u;
-    unsigned long long cap = hs.pairs;
-    if (a.chunk) cap += hs.pairs / 7 + (unsigned long long)warps * (a.chunk + hs.members);
-    a.cap = (unsigned)std::max<unsigned long long>(1, std::min(cap, kListMaxEntries));
+    auto room = [&](unsigned long long entries) {
+        return entries + (a.chunk ? entries / 7 + (unsigned long long)warps * (a.chunk + hs.members)
+                                  : 0ull);
+    };
+    unsigned long long cap = room(hs.pairs);
+    if (cap > limit) {
+        // The pairs bound the lists, but repeats may leave far less of them: a
+        // sample says how much.  An eighth of room for its error; lists that
+        // take more all the same end the build, and the net rounds color.
+        const int count = std::min(n, kListSample);
+        const size_t set = (size_t)wpb << (a.log + 2);
+        if (set > 48 * 1024)
+            PGC_CUDA(cudaFuncSetAttribute(net_list_sample,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set));
+        KernelTimer kt;
+        kt.prof = (o.flags & PGC_HOST_LOOP) ? o.profile : nullptr;
+        kt.stream = stream;
+        if (pgc_status s = kt.begin(2, "net_list_sample")) return s;
+        net_list_sample<<<(count + wpb - 1) / wpb, block, set, stream>>>(
+            dP, a.log, count, a.members <= (5 << a.log) / 8);
+        PGC_CUDA(cudaGetLastError());
+        if (pgc_status s = kt.end()) return s;
+        kt.destroy();
+        State* hs2 = cx.h_state.as<State>();
+        PGC_CUDA(cudaMemcpyAsync(hs2, cx.state.ptr, sizeof(State), cudaMemcpyDeviceToHost, stream));
+        PGC_CUDA(cudaStreamSynchronize(stream));
+        const double part = hs2->sample_pairs
+                                ? (double)hs2->sample_entries / (double)hs2->sample_pairs : 1.0;
+        const unsigned long long need = room((unsigned long long)((double)hs2->pairs * part));
+        if (need > limit) return PGC_OK;
+        cap = std::min(cap, std::min(limit, need + need / 8));
+    }
+    if (th.list_buffer) cap = std::min<unsigned long long>(cap, th.list_buffer);
+    a.cap = (unsigned)std::max<unsigned long long>(1, cap);
 
     const int bm_words = (hs.members >> 5) + 1;
     const d1::ScratchSizes z = d1::scratch_sizes(n, 0);
@@ -1414,7 +1494,6 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
     Opts lo = o;
     lo.mid_degree = kListMid;
     lo.hub_degree = 1 << kListMaxLog;
-    const Problem* dP = cx.problem.as<Problem>();
     const E::Setup setup = [&](const d1::Problem<d1::ListView>* dL) -> pgc_status {
         PGC_CUDA(cudaMemsetAsync(eng->live.ptr, 0xff, z.live, stream));
         PGC_CUDA(cudaMemsetAsync(eng->bm0.ptr, 0, z.bm0, stream));
@@ -1430,7 +1509,10 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
         return PGC_OK;
     }
     if (s != PGC_OK) return s;
-    if (eng->h_state.as<d1::State>()->status == d1::ST_LISTS) return PGC_OK;
+    if (eng->h_state.as<d1::State>()->status == d1::ST_LISTS) {
+        eng->release();
+        return PGC_OK;
+    }
     *taken = true;
     return eng->finish(lo, rounds, num_colors);
 }
@@ -1509,6 +1591,14 @@ static pgc_status run_scratch(Context& cx, const Input& in, int nnz, uint64_t se
     if (taken) {
         kt.destroy();
         return PGC_OK;
+    }
+    if (kt.prof) {   // the profile tells of the kernels that color
+        for (int k = 1; k < PGC_MAX_KERNELS; ++k) {
+            kt.prof->kernel_ms[k] = 0.0;
+            kt.prof->kernel_launches[k] = 0;
+            kt.prof->kernel_names[k] = nullptr;
+        }
+        kt.prof->num_kernels = kt.prof->num_launches = 1;
     }
     const long long need = (long long)hs->bound + 1;   // a first-fit color is <= |S(v)| + 1
     const int windows = (int)std::min<long long>(kMaxWindows, (need + 63) / 64);

@@ -241,4 +241,11 @@ pgc_status pgc_test_mid_barrier(uint32_t polls, int32_t slow_block, uint32_t slo
     return PGC_OK;
 }
 
+pgc_status pgc_test_list_room(uint32_t limit, uint32_t buffer) {
+    std::lock_guard<std::mutex> lk(pgc::g_hooks_mu);
+    pgc::g_hooks.list_limit = limit;
+    pgc::g_hooks.list_buffer = buffer;
+    return PGC_OK;
+}
+
 }  // extern "C"

@@ -53,6 +53,8 @@ struct TestHooks {
         unsigned slow_us = 0;       // ... by this many microseconds
         int at = 1;                 // ... at its at-th barrier (mid loop)
     } core, mid;                    // the core phase's meeting, the mid loop's barriers
+    unsigned list_limit = 0;        // conflict lists: entries they may take (0: the default)
+    unsigned list_buffer = 0;       // ... and the buffer gets at most this many (0: no limit)
 };
 TestHooks test_hooks();                 // a snapshot
 bool test_take_alloc_failure();         // true if this allocation must fail
