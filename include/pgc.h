@@ -108,7 +108,10 @@ typedef struct {
     /* per-round trace, entry r describes round r+1's worklist W_{r+1}:
        w[r] = |W_{r+1}|, s[r] = sum of deg(v), h[r] = sum of the lengths of
        the detection lists (neighbors, or for D2/PD2 vertices of a common net,
-       with higher priority; D2/PD2 in net rounds: the vertices' nets) */
+       with higher priority; D2/PD2 in net rounds: the vertices' nets).  A list
+       of D2/PD2 may name a vertex more than once where few would be repeated,
+       which depends on the device's size: w and s are the same everywhere, h
+       of D2/PD2 is not.  Entries past the last round are 0. */
     int64_t *trace_w;          /* host array of trace_cap entries, or NULL */
     int64_t *trace_s;          /* host array of trace_cap entries, or NULL */
     int64_t *trace_h;          /* host array of trace_cap entries, or NULL */

@@ -1514,6 +1514,11 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
         return PGC_OK;
     }
     *taken = true;
+    if (o.profile)   // no net is visited in any round
+        for (int i = 0; i < o.profile->trace_cap; ++i) {
+            if (o.profile->trace_nets) o.profile->trace_nets[i] = 0;
+            if (o.profile->trace_members) o.profile->trace_members[i] = 0;
+        }
     return eng->finish(lo, rounds, num_colors);
 }
 
