@@ -147,7 +147,9 @@ typedef struct {
     int32_t hub_degree;        /* D1; 0 => 16384: longer lists get a thread block */
     int32_t block;             /* 0 => default threads per block (128..1024) */
     int32_t grid_per_sm;       /* 0 => occupancy-derived blocks per SM */
-    int32_t timeout_ms;        /* 0 => 60000: device loop gives up after this */
+    int32_t timeout_ms;        /* 0 => 60000: device loop gives up after this,
+                                  looked at once a round; for D2/PD2 it covers
+                                  the build of the conflict lists, too */
     int32_t tail_vertices;     /* D1: once the worklist has at most this many
                                   vertices (4096 at most) and shrinks slowly,
                                   the remaining rounds run on the subgraph it

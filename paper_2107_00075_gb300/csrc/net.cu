@@ -999,6 +999,14 @@ __global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ 
     const unsigned lt = (1u << lane) - 1u;
     const long long gw = (long long)blockIdx.x * wpb + warp, nw = (long long)gridDim.x * wpb;
     const int self = P.self;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // the time limit covers the build
+        st->round = 1;
+        st->t0 = global_ns();
+        if (L.trace_cap > 0) {
+            L.trace_w[0] = P.n;
+            L.trace_s[0] = __ldg(P.r_ptr + P.n);
+        }
+    }
     unsigned at = 0u, end = 0u;   // this warp's part of the buffer
     unsigned long long my_h = 0ull, my_s = 0ull;
     bool full = false, few_repeats = false;
@@ -1183,14 +1191,6 @@ __global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ 
         if (my_s) atomicAdd(&st->s_next, my_s);
     }
     if (full && lane == 0) *(volatile int*)&st->lists_full = 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st->round = 1;
-        st->t0 = global_ns();
-        if (L.trace_cap > 0) {
-            L.trace_w[0] = P.n;
-            L.trace_s[0] = __ldg(P.r_ptr + P.n);
-        }
-    }
     d1::end_round1(L, st);
 }
 
