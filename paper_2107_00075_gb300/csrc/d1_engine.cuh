@@ -199,7 +199,7 @@ struct Hot {
     int nl[2];        // L-tier worklist sizes
     int push_cnt;     // push work items queued this round
     int max_color;
-    int stop;         // mid loop: round in which the time limit had passed (0: none)
+    int stop;         // mid loop: round before which the time limit had passed (0: none)
     int pend;         // round 1's queued pushes still wait (setup queues them)
     __host__ __device__ int count(int p) const { return ns[p] + nm[p] + nl[p]; }
 };
@@ -1377,7 +1377,8 @@ __global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp
         return grid_barrier(st, h, phase, P.mid_wait.polls);
     };
     int r = h.round, cur = h.count(r & 1), status = ST_OK, done = 0, tail = 0;
-    const unsigned long long t0 = lead ? st->t0 : 0ull;
+    const int first = r;   // (the round before it looked at the clock itself)
+    const unsigned long long t0 = lead ? st->t0 : 0ull, timeout_ns = P.timeout_ns;
     bool ok = true;
     if (h.pend && h.push_cnt > 0) {   // round 1's
         push_phase(P, h.push_cnt);
@@ -1385,16 +1386,18 @@ __global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp
     }
     while (ok) {
         const int np = (r & 1) ^ 1;
+        unsigned long long now = 0ull;
         if (lead) {
             st->push_cnt = 0;
             st->ns[np] = st->nm[np] = st->nl[np] = 0;
             st->s_next = st->h_next = 0ull;
-            // (a block may still be deciding the last round: hence the round number)
-            // the timer is slow to read: every eighth round
-            if ((r & 7) == 0 && global_ns() - t0 > P.timeout_ns && st->stop == 0) st->stop = r;
+            // the end of the last round; the timer is slow to read, so its value
+            // is used behind the barrier only
+            now = global_ns();
         }
         if (!DYN || r > 1) assign_phase(P, h, r);
         if (!barrier()) break;
+        if (lead && r > first && now - t0 > timeout_ns) st->stop = r;
         detect_phase<V, DYN>(P, h, r, smem);
         if (!barrier()) break;
         const int nxt = h.count(np), pushes = h.push_cnt;
@@ -1406,10 +1409,10 @@ __global__ void __launch_bounds__(T, 1) d1_mid(const Problem<V>* __restrict__ Pp
             }
             if (r == 1) P.trace_h[0] = (long long)st->h_first;
         }
-        if (nxt == 0) done = 1;
+        if (h.stop) status = ST_TIMEOUT;   // passed before this round began
+        else if (nxt == 0) done = 1;
         else if (nxt >= cur) status = ST_NO_PROGRESS;
         else if (r >= P.max_rounds) status = ST_MAX_ROUNDS;
-        else if (h.stop > 0 && h.stop <= r) status = ST_TIMEOUT;
         if (done || status != ST_OK) break;
         tail = nxt <= P.tail_w && (long long)(cur - nxt) * kCoreRounds < nxt;
         cur = nxt;
@@ -1922,6 +1925,9 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
     const bool go = X.gave_up == 0;
     while (go) {
         const int now = r & 1, old = now ^ 1;
+        // the end of the last round; the timer is slow to read, so its value is
+        // used behind the cluster barrier only
+        const unsigned long long at_ns = cta == 0 && tid == 0 ? global_ns() : 0ull;
         const int n_open = X.n_open[now];
         uint4* const won = S.won + old * words4;
         unsigned short* const open = S.open + now * S.R;
@@ -1982,8 +1988,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
             X.moved = 0u;
             X.n_open[old] = 0;
             X.n_won[old] = 0u;
-            // the timer is slow to read: every 16th round
-            if (cta == 0 && (r & 15) == 0 && global_ns() - t0_ns > timeout_ns)
+            if (cta == 0 && at_ns - t0_ns > timeout_ns)
                 for (int c = 0; c < C; ++c) st_peer(peer_u32(&X.stop, c), 1u);
         }
         for (int i = tid; i < words4; i += kCoreThreads) won[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -2064,10 +2069,10 @@ __global__ void __launch_bounds__(kCoreThreads, 1) d1_core_loop(const Problem<V>
                 P.trace_h[r] = (long long)th;
             }
         }
-        if (nxt == 0) break;
-        if (n_won == 0) status = ST_NO_PROGRESS;
+        if (X.stop) status = ST_TIMEOUT;   // passed before this round began
+        else if (nxt == 0) break;
+        else if (n_won == 0) status = ST_NO_PROGRESS;
         else if (r >= max_rounds) status = ST_MAX_ROUNDS;
-        else if (X.stop) status = ST_TIMEOUT;
         if (status != ST_OK) break;
         cur = nxt;
         ++r;
