@@ -2116,7 +2116,14 @@ struct Scratch {
     int2* items;
     int2* pushq;
     int* prio = nullptr;   // n ints, only for priorities that change each round
+    unsigned* core_mat = nullptr;   // core_mat_bytes(n); none: no core phase
 };
+
+// The core phase's adjacency bits: a worklist of k vertices takes k x ceil(k / 32) words.
+inline size_t core_mat_bytes(long long n) {
+    const size_t k = (size_t)std::min<long long>(n, kCoreMax);
+    return k * ((k + 31) / 32) * 4;
+}
 
 struct ScratchSizes {
     size_t deg, hlen, hadj, bm0, bmx, live, list, items, pushq;
@@ -2502,6 +2509,8 @@ struct Engine {
         sc.items = items.as<int2>();
         sc.pushq = pushq.as<int2>();
         sc.prio = varying ? prio.as<int>() : nullptr;
+        if (pgc_status s = core_mat.ensure(core_mat_bytes(n))) return s;
+        sc.core_mat = core_mat.as<unsigned>();
         if (pgc_status s = launch(sc, view, n, nnz, d_col, g_rounds, g_colors, seed, o, stream,
                                   up))
             return s;
@@ -2544,8 +2553,6 @@ struct Engine {
         last_want_trace = want_trace;
         last_tcap = tcap;
 
-        const int core_k = std::min(n, kCoreMax);
-        if (pgc_status s = core_mat.ensure((size_t)core_k * ((core_k + 31) / 32) * 4)) return s;
         Geometry g;
         if (pgc_status s = geometry(o, &g)) return s;
 
@@ -2566,7 +2573,7 @@ struct Engine {
         }
         hp->items = sc.items;
         hp->push_q = sc.pushq;
-        hp->core_mat = core_mat.as<unsigned>();
+        hp->core_mat = sc.core_mat;
         hp->g_rounds = g_rounds;
         hp->g_colors = g_colors;
         hp->trace_w = trace.as<long long>();
@@ -2589,7 +2596,7 @@ struct Engine {
         hp->det_m = pflags ? std::max(o.mid_degree, std::min(o.hub_degree, varying_hub((int)n)))
                            : o.hub_degree;
         hp->mid_w = hp->async_mode || g.mid_grid == 0 ? 0 : shares_gpu ? kMidSharedMax : kMidMax;
-        hp->tail_w = hp->mid_w == 0 || pflags || g.core_grid == 0
+        hp->tail_w = hp->mid_w == 0 || pflags || g.core_grid == 0 || !sc.core_mat
                          ? 0 : std::min(o.tail_vertices, kCoreMax);
         const int small = n <= hp->mid_w ? 2 : 0;
         const TestHooks th = test_hooks();

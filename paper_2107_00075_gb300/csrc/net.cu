@@ -1473,6 +1473,7 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
     need(eng->wm, z.list);
     need(eng->wl, z.list);
     need(eng->pushq, ((size_t)n + a.cap / d1::kPushItem + 1) * sizeof(int2));
+    need(eng->core_mat, d1::core_mat_bytes(n));
     if (s == PGC_ERR_OOM) {
         eng->release();
         return PGC_OK;
@@ -1490,6 +1491,7 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
     sc.wm = eng->wm.as<int4>();
     sc.wl = eng->wl.as<int4>();
     sc.pushq = eng->pushq.as<int2>();
+    sc.core_mat = eng->core_mat.as<unsigned>();
     d1::ListView view{a.rows, a.lists, in.r_ptr, bm_words};
     Opts lo = o;
     lo.mid_degree = kListMid;

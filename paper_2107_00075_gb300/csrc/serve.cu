@@ -52,6 +52,7 @@ struct Request {
     uint64_t seed = 1;
     int windows = 1;
     size_t bytes = 0, off = 0;
+    size_t core_bytes = 0;        // ... of bytes, the last: the core phase's (0: it does without)
     int slot = -1;
     bool done = false;
     pgc_status status = PGC_OK;
@@ -102,7 +103,7 @@ struct Server {
     std::string engine_error;
 };
 
-// Device bytes a request needs while it is active.
+// Device bytes a request needs while it is active (the core phase's apart).
 static size_t footprint(const Request& r) {
     if (r.kind == KIND_D1) {
         return al((size_t)(r.n + 1) * 4) + al((size_t)std::max<long long>(r.nnz, 1) * 4) +
@@ -132,6 +133,7 @@ static pgc_status start(Server& S, Slot& sl, Request& r) {
         if (r.nnz)
             PGC_CUDA(cudaMemcpyAsync(d_ci, r.ci, (size_t)r.nnz * 4, cudaMemcpyDefault, st));
         d1::Scratch sc = d1::carve_scratch(p, r.n, r.nnz);
+        if (r.core_bytes) sc.core_mat = reinterpret_cast<unsigned*>(base + r.bytes - r.core_bytes);
         Opts o;
         if (pgc_status s = sl.d1e.launch(sc, d1::SingleView{d_rp, d_ci}, r.n, r.nnz, d_col,
                                          nullptr, nullptr, r.seed, o, st))
@@ -284,6 +286,11 @@ static pgc_status submit(Server* S, Request* r, long long* req_id) {
         delete r;
         return fail(PGC_ERR_BUSY, "request footprint exceeds the server's HBM budget");
     }
+    // the core phase saves time, not memory: a request that fits the budget
+    // only without it is colored without it
+    if (r->kind == KIND_D1) r->core_bytes = al(d1::core_mat_bytes(r->n));
+    if (r->bytes + r->core_bytes > S->budget) r->core_bytes = 0;
+    r->bytes += r->core_bytes;
     r->id = S->next_id++;
     S->reqs[r->id] = r;
     S->queue.push_back(r);
