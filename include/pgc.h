@@ -35,7 +35,10 @@
  * memory (staged through library-owned device buffers; the call then also
  * copies the colors back).  The library never frees caller memory.  Scratch
  * (degrees, worklists, masks, counters) is library-owned, allocated on
- * first use per device and reused; pgc_release() frees it.
+ * first use per device and reused; pgc_release() frees it.  Distance-2
+ * colorings keep their conflict lists' buffers in the same way (2 GB of lists
+ * at most); any call that runs out of device memory frees these and tries once
+ * more before it returns PGC_ERR_OOM.
  *
  * Threads and streams: calls on one device are serialized by the library;
  * `stream` (a cudaStream_t, NULL = the legacy default stream) orders the
@@ -371,8 +374,10 @@ const char *pgc_version(void);
  *
  * pgc_test_fail_alloc(after): the device allocation the library attempts
  *   after `after` further successful ones fails as if the device were out of
- *   memory, once; the call that meets it returns PGC_ERR_OOM having freed
- *   the scratch of that engine.  after < 0 disarms.
+ *   memory, once.  The call that meets it returns PGC_ERR_OOM having freed
+ *   the scratch of that engine, except that D2/PD2 colors in net rounds when
+ *   the buffers of its conflict lists fail, and that a call which finds
+ *   conflict lists of an earlier one to free goes on.  after < 0 disarms.
  * pgc_test_core_barrier(polls, slow_block, slow_us): the blocks of the core
  *   loop (the last rounds, one thread-block cluster) meet before its first
  *   round; the meeting gives up after `polls` polls (0: the default, about one

@@ -301,8 +301,10 @@ extern "C" pgc_status pgc_color_d1_batch(int32_t G, const int64_t* vtx_off, cons
                                          int32_t* ncolors_per_g, int32_t* rounds,
                                          const pgc_opts* opts, void* stream) {
     try {
-        return pgc::d1::color_batch(G, vtx_off, nnz_off, row_ptr, col_idx, seed, colors,
-                                    rounds_per_g, ncolors_per_g, rounds, opts, stream);
+        return pgc::or_without_lists([&] {
+            return pgc::d1::color_batch(G, vtx_off, nnz_off, row_ptr, col_idx, seed, colors,
+                                        rounds_per_g, ncolors_per_g, rounds, opts, stream);
+        });
     } catch (const std::exception& e) {
         return pgc::fail(PGC_ERR_CUDA, e.what());
     } catch (...) {

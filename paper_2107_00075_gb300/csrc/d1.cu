@@ -123,7 +123,10 @@ extern "C" pgc_status pgc_color_d1(int32_t n, const int32_t* row_ptr, const int3
                                    uint64_t seed, int32_t* colors, int32_t* rounds,
                                    int32_t* num_colors, const pgc_opts* opts, void* stream) {
     try {
-        return pgc::d1::color(n, row_ptr, col_idx, seed, colors, rounds, num_colors, opts, stream);
+        return pgc::or_without_lists([&] {
+            return pgc::d1::color(n, row_ptr, col_idx, seed, colors, rounds, num_colors, opts,
+                                  stream);
+        });
     } catch (const std::exception& e) {
         return pgc::fail(PGC_ERR_CUDA, e.what());
     } catch (...) {

@@ -1914,8 +1914,10 @@ extern "C" pgc_status pgc_color_d2(int32_t n, const int32_t* row_ptr, const int3
                                    uint64_t seed, int32_t* colors, int32_t* rounds,
                                    int32_t* num_colors, const pgc_opts* opts, void* stream) {
     try {
-        return pgc::net::color(2, n, n, row_ptr, col_idx, nullptr, nullptr, seed, colors, rounds,
-                               num_colors, opts, stream);
+        return pgc::or_without_lists([&] {
+            return pgc::net::color(2, n, n, row_ptr, col_idx, nullptr, nullptr, seed, colors,
+                                   rounds, num_colors, opts, stream);
+        });
     } catch (const std::exception& e) {
         return pgc::fail(PGC_ERR_CUDA, e.what());
     } catch (...) {
@@ -1929,8 +1931,10 @@ extern "C" pgc_status pgc_color_pd2(int32_t n_rows, int32_t n_cols, const int32_
                                     int32_t* rounds, int32_t* num_colors, const pgc_opts* opts,
                                     void* stream) {
     try {
-        return pgc::net::color(3, n_rows, n_cols, row_ptr, col_idx, col_ptr, row_idx, seed, colors,
-                               rounds, num_colors, opts, stream);
+        return pgc::or_without_lists([&] {
+            return pgc::net::color(3, n_rows, n_cols, row_ptr, col_idx, col_ptr, row_idx,
+                                   seed, colors, rounds, num_colors, opts, stream);
+        });
     } catch (const std::exception& e) {
         return pgc::fail(PGC_ERR_CUDA, e.what());
     } catch (...) {
@@ -1945,8 +1949,10 @@ extern "C" pgc_status pgc_color_pd2_bipartite(int32_t n_rows, int32_t n_cols,
                                                int32_t* num_colors, const pgc_opts* opts,
                                                void* stream) {
     try {
-        return pgc::net::color(4, n_rows, n_cols, row_ptr, col_idx, col_ptr, row_idx, seed, colors,
-                               rounds, num_colors, opts, stream);
+        return pgc::or_without_lists([&] {
+            return pgc::net::color(4, n_rows, n_cols, row_ptr, col_idx, col_ptr, row_idx,
+                                   seed, colors, rounds, num_colors, opts, stream);
+        });
     } catch (const std::exception& e) {
         return pgc::fail(PGC_ERR_CUDA, e.what());
     } catch (...) {
@@ -1982,6 +1988,16 @@ pgc_status slot_launch_pd2(void* c, void* scratch, int n_rows, int n_cols, const
     in.col = colors;
     Opts o;
     return launch_known(*cx, scratch, in, windows, seed, o, stream);
+}
+
+bool release_lists() {
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    auto* eng = d1::engine_for<d1::ListView>(device);
+    std::unique_lock<std::mutex> lk(eng->mu, std::try_to_lock);
+    if (!lk.owns_lock() || !eng->hadj.ptr) return false;
+    eng->release();
+    return true;
 }
 
 bool slot_overflowed(void* c) {

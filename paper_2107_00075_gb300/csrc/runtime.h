@@ -102,8 +102,12 @@ pgc_status csr_csc_pair(const int* rp, const int* ci, int n_rows, const int* cp,
                         int n_cols, const DeviceInfo& dev, cudaStream_t stream);
 }  // namespace validate
 
-// Partial distance-2 engine slots for the server (net.cu).
+// Partial distance-2 engine slots for the server, and the memory that the
+// conflict lists of the last distance-2 coloring keep for the next (net.cu).
 namespace net {
+// Frees the lists on the current device; false if there are none, or if a call
+// on another thread is using them.
+bool release_lists();
 size_t scratch_bytes(int n, int n_nets, int windows);
 void* slot_create();
 void slot_destroy(void* slot);
@@ -113,5 +117,12 @@ pgc_status slot_launch_pd2(void* slot, void* scratch, int n_rows, int n_cols, co
 pgc_status slot_finish(void* slot, int* rounds, int* num_colors);
 bool slot_overflowed(void* slot);   // the last launch needed more mask windows
 }  // namespace net
+
+// f(), and once more if it met PGC_ERR_OOM and the conflict lists could be freed.
+template <class F>
+pgc_status or_without_lists(F f) {
+    const pgc_status s = f();
+    return s == PGC_ERR_OOM && net::release_lists() ? f() : s;
+}
 
 }  // namespace pgc

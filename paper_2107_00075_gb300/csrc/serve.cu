@@ -348,7 +348,8 @@ pgc_status pgc_server_create(size_t hbm_budget_bytes, int32_t max_active, pgc_se
             return pgc::fail(PGC_ERR_CUDA, "no current device");
         }
         S.budget = hbm_budget_bytes;
-        if (pgc_status s = S.arena_mem.ensure(hbm_budget_bytes)) {
+        if (pgc_status s = pgc::or_without_lists(
+                [&] { return S.arena_mem.ensure(hbm_budget_bytes); })) {
             delete srv;
             return s;
         }

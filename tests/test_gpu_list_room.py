@@ -158,3 +158,35 @@ def test_net_rounds_in_every_launch_form(pgc, kw, host_loop):
     for x in WIDE:
         names = color(pgc, x, flags=pgc.PGC_HOST_LOOP if host_loop else 0, **kw)
         assert not host_loop or ("net_detect" in names and "net_lists" not in names)
+
+
+def test_any_call_takes_the_lists_memory_when_out_of_its_own(pgc):
+    """The lists that a D2 call left are freed for a D1, batched or D2 call that
+    meets an out-of-memory, which then succeeds; without them it reports it."""
+    g, wide = gen.rmat(10, 8, seed=5), gen.stencil3d(30, 30, 30, points=7)
+    d1 = oracle.color_d1(g.row_ptr, g.col_idx, seed=1)
+    batch = gen.make_batch([g, g])
+    calls = {
+        "d1": lambda: pgc.pgc_color_d1(dev(g.row_ptr), dev(g.col_idx)).colors.cpu().numpy(),
+        "batch": lambda: pgc.pgc_color_d1_batch(
+            batch.vtx_off, batch.nnz_off, batch.row_ptr, batch.col_idx).colors[:g.n],
+        "d2": lambda: pgc.pgc_color_d2(dev(wide.row_ptr), dev(wide.col_idx), seed=2
+                                       ).colors.cpu().numpy(),
+    }
+    expect = {"d1": d1.colors, "batch": d1.colors, "d2": wanted(wide).colors}
+    for name, call in calls.items():
+        for held in (True, False):
+            pgc.pgc_release()
+            if held:
+                assert "net_lists" in color(pgc, PATTERN)
+            pgc.pgc_test_fail_alloc(0)
+            try:
+                if held:
+                    assert np.array_equal(call(), expect[name]), name
+                else:
+                    with pytest.raises(pgc.PgcError) as e:
+                        call()
+                    assert e.value.status == 3, name
+            finally:
+                pgc.pgc_test_fail_alloc(-1)
+            assert np.array_equal(call(), expect[name]), name
