@@ -2333,20 +2333,22 @@ struct Engine {
         return k;
     }
 
-    pgc_status build_graph(const Geometry& g, int async, int dyn) {
-        destroy_graph();
-        for (int k = 0; k < kGraphs; ++k) {
-            const bool setup = k % 2 == 0, small = k >= 2;
-            if ((setup && !V::kSetup) || (small && (async || g.mid_grid == 0))) continue;
-            if (pgc_status s = build_one_graph(g, setup, small, async, dyn, &graph[k], &exec[k]))
-                return s;
+    // Graph k for this geometry and mode, built when a call first needs it (the
+    // four together take 0.05 ms of a first call's 0.48).
+    pgc_status ensure_graph(int k, const Geometry& g, int async, int dyn) {
+        if (g_grid != g.grid || g_block != g.block || g_det != g.det_grid || g_async != async ||
+            g_dyn != dyn) {
+            destroy_graph();
+            g_dyn = dyn;
+            g_grid = g.grid;
+            g_det = g.det_grid;
+            g_block = g.block;
+            g_async = async;
         }
-        g_dyn = dyn;
-        g_grid = g.grid;
-        g_det = g.det_grid;
-        g_block = g.block;
-        g_async = async;
-        return PGC_OK;
+        if (exec[k]) return PGC_OK;
+        if (graph[k]) cudaGraphDestroy(graph[k]);   // of a call that failed
+        graph[k] = nullptr;
+        return build_one_graph(g, k % 2 == 0, k >= 2, async, dyn, &graph[k], &exec[k]);
     }
 
     // Setup (optional, with round 1), round 1 when it is not part of the setup
@@ -2608,17 +2610,15 @@ struct Engine {
 
         State* hs = h_state.as<State>();
         if (!(o.flags & PGC_HOST_LOOP)) {
-            const int dyn = hp->prio_mode != 0;
-            if (!exec[1] || g_grid != g.grid || g_block != g.block || g_det != g.det_grid ||
-                g_async != hp->async_mode || g_dyn != dyn) {
-                if (pgc_status s = build_graph(g, hp->async_mode, dyn)) return s;
-            }
+            const int which = !V::kSetup ? small + 1 : up ? 1 : small;
+            if (pgc_status s = ensure_graph(which, g, hp->async_mode, hp->prio_mode != 0))
+                return s;
             if constexpr (!V::kSetup) {
                 PGC_CUDA(cudaMemsetAsync(state.ptr, 0, sizeof(State), stream));
                 if (pgc_status s = (*setup)(dP)) return s;
-                PGC_CUDA(cudaGraphLaunch(exec[small + 1], stream));
+                PGC_CUDA(cudaGraphLaunch(exec[which], stream));
             } else if (!up) {
-                PGC_CUDA(cudaGraphLaunch(exec[small], stream));
+                PGC_CUDA(cudaGraphLaunch(exec[which], stream));
             } else {
                 // setup by hand: classify needs only the row offsets; the
                 // build of row range k waits for that range's copy
@@ -2653,7 +2653,7 @@ struct Engine {
                 }
                 d1_tier<V><<<g.grid, g.block, 0, stream>>>(dP, state.as<State>());
                 PGC_CUDA(cudaGetLastError());
-                PGC_CUDA(cudaGraphLaunch(exec[1], stream));
+                PGC_CUDA(cudaGraphLaunch(exec[which], stream));
             }
         } else {
             KernelTimer kt;
