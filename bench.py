@@ -186,7 +186,7 @@ def d1_setup_bytes(n, nnz, h1, deg=None, build_item=512, build_m=512):
     }
 
 
-def d1_round_bytes(trace_w, trace_s, trace_h):
+def d1_round_bytes(trace_w, trace_s, trace_h, whole_lists=True):
     """Per-round bytes of the three round kernels, from the trace (entry r-1
     describes round r: |W_r|, S_r = sum of deg over W_r, H_r = sum of the
     priority-list lengths over W_r).  Returns three arrays (one entry per
@@ -195,8 +195,11 @@ def d1_round_bytes(trace_w, trace_s, trace_h):
                 write 4 = 32 per worklist vertex (overflow-bitmap words of
                 vertices past color 64 not counted)
       detect:   entry 16 + own color 4 per worklist vertex; 8 per priority-list
-                entry (id + the neighbor's color; round 1 reads no list; an
-                upper bound, losers stop at their first conflict); per winner
+                entry read (id + the neighbor's color; round 1 reads no list):
+                every entry of the worklist's lists with whole_lists, an upper
+                bound, since losers stop at their first conflict; else what is
+                read at least, the winners' lists (H_r - H_{r+1}) and the first
+                step of the losers', four entries or the mean list; per winner
                 a color write and an uncolored-bit update (8) and its push
                 items (8 per 128 adjacency entries); per loser its next-round
                 entry (16)
@@ -213,6 +216,9 @@ def d1_round_bytes(trace_w, trace_s, trace_h):
     if len(asg):
         asg[0] = 0.0
     lists = hh.copy()
+    if not whole_lists:
+        hn = np.append(hh[1:], 0.0)
+        lists = hh - hn + np.minimum(4.0 * wn, hn)
     if len(lists):
         lists[0] = 0.0
     det = 20.0 * w + 8.0 * lists + 8.0 * won + won_adj / 16.0 + 16.0 * wn
@@ -262,7 +268,8 @@ def d1_algorithmic_bytes(trace_w, trace_s, trace_h, n, nnz, tail_at=None, deg=No
 
 
 MID_W = 65536    # worklists up to this size: the rounds run in one launch (d1_mid)
-CORE_W = 4096    # ... and, while they shrink slowly, in the core phase (d1_core)
+CORE_W = 4096    # ... and, while they shrink by less than 1 / CORE_PACE a round, in
+CORE_PACE = 8    # the core phase (d1_core)
 
 
 def d1_phases(prof):
@@ -277,14 +284,15 @@ def d1_phases(prof):
     core = R
     if "d1_core" in prof.kernel_ms:
         core = next((i for i in range(mid + 1, R)
-                     if w[i] <= CORE_W and (w[i - 1] - w[i]) * 8 < w[i]), R)
+                     if w[i] <= CORE_W and (w[i - 1] - w[i]) * CORE_PACE < w[i]), R)
     return mid, core
 
 
 def d1_phase_bytes(prof, setup, last_setup, row_mean=None):
     """Bytes each kernel of a profiled coloring moves: the setup kernels'
     (setup; round 1 runs in last_setup), then the per-round model of
-    d1_round_bytes split over the launched rounds, d1_mid and the core phase.
+    d1_round_bytes (the list entries that are read at least) split over the
+    launched rounds, d1_mid and the core phase.
     The core phase's rounds stay in shared memory: it reads, per entry of its
     worklist's lists, the id, its uncolored word and its rank (12), and per
     vertex its entry, color and key (28).  row_mean: entries a winner pushes
@@ -292,7 +300,7 @@ def d1_phase_bytes(prof, setup, last_setup, row_mean=None):
     mid, core = d1_phases(prof)
     w = np.asarray(prof.trace_w, dtype=np.float64)
     sw = prof.trace_s if row_mean is None else row_mean * w
-    asg, det, psh = d1_round_bytes(w, sw, prof.trace_h)
+    asg, det, psh = d1_round_bytes(w, sw, prof.trace_h, whole_lists=False)
     nb = dict(setup)
     if len(w):
         nb[last_setup] += float(det[0] + psh[0])
