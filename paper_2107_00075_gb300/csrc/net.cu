@@ -16,7 +16,8 @@
 // Conflict lists (net_lists): the vertices that share a net with v, each once,
 // are its row in the conflict graph, and the distance-1 engine runs the
 // rounds.  The way of every problem whose vertices have fewer than 2048
-// members in their nets and whose lists fit 2 GB.
+// members in their nets and whose lists fit 2 GB, but for large problems with
+// little per vertex (net_rounds_pay).
 //
 // Net rounds, for the others.  Per round:
 //   assign  v in W: forbidden(v) = OR of the color masks of v's nets;
@@ -59,7 +60,7 @@ struct State {
     int all_active;   // this round every net is treated as active (no marking)
     unsigned blocks_done;
     int bound;        // max over v of sum over its nets of (|net| - 1)
-    int pad;
+    int max_net;      // members of the largest net of a vertex
     unsigned long long s_next;
     unsigned long long h_next;
     unsigned long long h_first;
@@ -133,7 +134,7 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
     const int warp = threadIdx.x >> 5;
     WarpAppend at = {smem + warp * 2 * kAppendSlots, 0},
                aw = {smem + warp * 2 * kAppendSlots + kAppendSlots, 0};
-    int my_bound = 0, my_deg = 0, my_members = 0;
+    int my_bound = 0, my_deg = 0, my_members = 0, my_net = 0;
     unsigned long long my_h = 0ull, my_pairs = 0ull;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long wbase = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
@@ -151,7 +152,11 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
             my_deg = max(my_deg, d);
             k = d + P.self;
             long long b = 0;
-            for (int j = 0; j < k; ++j) b += net_size(P, vertex_net(P, v, beg, j)) - 1;
+            for (int j = 0; j < k; ++j) {
+                const int size = net_size(P, vertex_net(P, v, beg, j));
+                b += size - 1;
+                my_net = max(my_net, size);
+            }
             my_bound = max(my_bound, (int)min(b, (long long)INT32_MAX - 1));
             my_pairs += (unsigned long long)b;
             my_members = max(my_members, (int)min(b + k, (long long)INT32_MAX - 1));
@@ -169,7 +174,9 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
     my_h = warp_sum(my_h);
     my_pairs = warp_sum(my_pairs);
     my_members = warp_max(my_members);
+    my_net = warp_max(my_net);
     if (lane_id() == 0) {
+        atomicMax(&st->max_net, my_net);
         if (my_pairs) atomicAdd(&st->pairs, my_pairs);
         atomicMax(&st->bound, my_bound);
         atomicMax(&st->members, my_members);
@@ -1385,22 +1392,40 @@ static pgc_status run(Context& cx, const Input& in, int nnz, uint64_t seed, cons
     return s;
 }
 
+// Large problems with little to look at per vertex are faster in net rounds: the
+// lists cost a build, and what they save is the latency of the rounds' three
+// launches (many rounds of small worklists) and visits of whole nets (many
+// members).  Lists against net rounds, ms, by vertices and mean pairs per vertex
+// (a member of a net of a vertex other than the vertex):
+//   0.5M: 41 pairs 1.05 / 1.24 (7-point mesh), 20 0.79 / 0.84 (grid), 8 0.84 / 1.13 (PD2)
+//   1M:   41 1.67 / 1.72, 20 1.24 / 1.11, PD2 16 1.58 / 1.53, 47 2.99 / 2.79, 79 3.91 / 4.52
+//   2M:   41 3.50 / 2.97, 20 2.23 / 1.76, PD2 31 3.71 / 3.29, 63 5.71 / 5.87, 79 6.92 / 7.56
+//   4M:   PD2 16 5.58 / 3.50, 63 11.1 / 10.6; D2 of random graphs 80 12.7 / 11.7
+//   16M:  41 22.2 / 21.9, 24 27.0 / 23.5, 20 16.0 / 11.4; PD2 4 10.8 / 5.3
+// The line of equal times grows with the vertices (48 pairs at 1M, 64 at 2M, 96 at
+// 4M).  All measured nets fit a warp; one longer than that means as many rounds
+// as it has members, and those are what the lists are for.
+static bool net_rounds_pay(int n, const State& hs) {
+    return n >= 1000000 && hs.max_net <= 32 && hs.members <= 512 &&
+           hs.pairs < (unsigned long long)n * (32u + (unsigned)n / 65536u);
+}
+
 // The coloring as a distance-1 coloring of the conflict graph, once net_init
 // has run and hs holds its sums.  *taken is false when the problem is left to
-// the net rounds: a vertex with too many members for a warp's set, lists that
-// would not fit kListMaxEntries, or no device memory for them.  The net rounds
-// then find the memory that the lists held free again.
+// the net rounds: they are faster, a vertex has too many members for a warp's
+// set, the lists would not fit kListMaxEntries, or there is no device memory for
+// them.  The net rounds then find the memory that the lists held free again.
 static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& hs, uint64_t seed,
                             const Opts& o, cudaStream_t stream, int* rounds, int* num_colors,
                             bool* taken) {
     using E = d1::Engine<d1::ListView>;
     *taken = false;
     const int n = in.n;
-    if (hs.members >= 1 << kListMaxLog) return PGC_OK;
+    const TestHooks th = test_hooks();
+    if (hs.members >= 1 << kListMaxLog || (!th.list_limit && net_rounds_pay(n, hs))) return PGC_OK;
     E* eng = d1::engine_for<d1::ListView>(cx.dev.device);
     std::lock_guard<std::mutex> lk(eng->mu);
     eng->dev = cx.dev;
-    const TestHooks th = test_hooks();
     const unsigned long long limit = th.list_limit ? th.list_limit : kListMaxEntries;
 
     ListArgs a = {};

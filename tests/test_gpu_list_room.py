@@ -190,3 +190,62 @@ def test_any_call_takes_the_lists_memory_when_out_of_its_own(pgc):
             finally:
                 pgc.pgc_test_fail_alloc(-1)
             assert np.array_equal(call(), expect[name]), name
+
+
+def _small_nets(n):
+    """Columns 2i and 2i + 1 in one row each, every tenth row twice."""
+    a = np.arange(0, n - n % 2, 2)
+    rows = np.stack([a, a + 1], 1)
+    return _equal_rows(np.concatenate([rows, rows[::10]]), n)
+
+
+def _blocks(n):
+    """Rows of 32 neighbors, at every 16th column."""
+    return _equal_rows((np.arange(0, n - 31, 16)[:, None] + np.arange(32)), n)
+
+
+def _equal_rows(rows, n):
+    count, length = rows.shape
+    row_ptr = np.arange(0, length * count + 1, length, dtype=np.int32)
+    col_idx = rows.reshape(-1).astype(np.int32)
+    order = np.argsort(col_idx, kind="stable")
+    col_ptr = np.zeros(n + 1, np.int32)
+    col_ptr[1:] = np.cumsum(np.bincount(col_idx, minlength=n))
+    return gen.Bipartite(count, n, row_ptr, col_idx, col_ptr, (order // length).astype(np.int32))
+
+
+def _plus_row(b, members):
+    """b and one more row of the first columns."""
+    extra = np.arange(members, dtype=np.int32)
+    row_ptr = np.append(b.row_ptr, b.row_ptr[-1] + members).astype(np.int32)
+    col_idx = np.append(b.col_idx, extra)
+    at = np.repeat(np.arange(b.n_rows + 1), np.diff(row_ptr))
+    order = np.argsort(col_idx, kind="stable")
+    col_ptr = np.zeros(b.n_cols + 1, np.int32)
+    col_ptr[1:] = np.cumsum(np.bincount(col_idx, minlength=b.n_cols))
+    return gen.Bipartite(b.n_rows + 1, b.n_cols, row_ptr, col_idx, col_ptr,
+                         at[order].astype(np.int32))
+
+
+# Which way colors: the number of vertices (1,000,000 or more), the mean pairs per
+# vertex (fewer than 47 there) and the largest net (32 at most) decide.
+@pytest.mark.parametrize("make,lists", [
+    (lambda: _small_nets(999_999), True),
+    (lambda: _small_nets(1_000_000), False),
+    (lambda: _small_nets(1_200_001), False),
+    (lambda: _plus_row(_small_nets(1_000_000), 32), False),
+    (lambda: _plus_row(_small_nets(1_000_000), 33), True),
+    (lambda: gen.stencil3d(110, 110, 110, points=7), False),   # 41.3 pairs, the line at 52.3
+    (lambda: _blocks(1_000_000), True),    # 62 pairs, the line at 47.3
+], ids=["999999", "1000000", "1200001", "net of 32", "net of 33", "mesh", "blocks"])
+def test_large_problems_with_little_per_vertex_take_net_rounds(pgc, make, lists):
+    x = make()
+    names = color(pgc, x)
+    assert ("net_lists" in names, "net_detect" in names) == (lists, not lists)
+    color(pgc, x, flags=0)
+    pgc.pgc_test_list_room(1 << 30 if not lists else 1, 0)   # the other way, same colors
+    try:
+        names = color(pgc, x)
+        assert ("net_lists" in names, "net_detect" in names) == (not lists, lists)
+    finally:
+        pgc.pgc_test_list_room(0, 0)
