@@ -17,7 +17,7 @@
 // are its row in the conflict graph, and the distance-1 engine runs the
 // rounds.  The way of every problem whose vertices have fewer than 2048
 // members in their nets and whose lists fit 2 GB, but for large problems with
-// little per vertex (net_rounds_pay).
+// few nets per vertex (net_rounds_pay).
 //
 // Net rounds, for the others.  Per round:
 //   assign  v in W: forbidden(v) = OR of the color masks of v's nets;
@@ -37,6 +37,7 @@
 #include "d1_engine.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <functional>
 #include <memory>
@@ -1392,22 +1393,26 @@ static pgc_status run(Context& cx, const Input& in, int nnz, uint64_t seed, cons
     return s;
 }
 
-// Large problems with little to look at per vertex are faster in net rounds: the
-// lists cost a build, and what they save is the latency of the rounds' three
-// launches (many rounds of small worklists) and visits of whole nets (many
-// members).  Lists against net rounds, ms, by vertices and mean pairs per vertex
-// (a member of a net of a vertex other than the vertex):
-//   0.5M: 41 pairs 1.05 / 1.24 (7-point mesh), 20 0.79 / 0.84 (grid), 8 0.84 / 1.13 (PD2)
-//   1M:   41 1.67 / 1.72, 20 1.24 / 1.11, PD2 16 1.58 / 1.53, 47 2.99 / 2.79, 79 3.91 / 4.52
-//   2M:   41 3.50 / 2.97, 20 2.23 / 1.76, PD2 31 3.71 / 3.29, 63 5.71 / 5.87, 79 6.92 / 7.56
-//   4M:   PD2 16 5.58 / 3.50, 63 11.1 / 10.6; D2 of random graphs 80 12.7 / 11.7
-//   16M:  41 22.2 / 21.9, 24 27.0 / 23.5, 20 16.0 / 11.4; PD2 4 10.8 / 5.3
-// The line of equal times grows with the vertices (48 pairs at 1M, 64 at 2M, 96 at
-// 4M).  All measured nets fit a warp; one longer than that means as many rounds
-// as it has members, and those are what the lists are for.
+// Large problems with few nets per vertex are faster in net rounds: a round visits
+// the worklist's nets, k of them per vertex, while lists cost a build and a search
+// over the pairs, k r of them (r: the other members of a vertex's net, mean).  What
+// the lists save on small problems is the latency of a round's three launches.
+// Lists / net rounds in ms, patterns with rows of one mean length, by k:
+//   n = 1M: r 3.7: 4 1.60 / 1.47, 6 1.86 / 1.97;   r 7.9: 6 2.99 / 2.79, 10 3.91 / 4.52
+//           r 15: 4 3.19 / 2.59, 12 7.74 / 7.96;   r 26: 4 5.56 / 3.60, 16 18.0 / 18.3
+//   n = 2M: r 3.7: 4 2.76 / 2.31, 8 3.49 / 4.20;   r 10.9: 8 8.31 / 6.94, 16 14.8 / 17.0
+//   n = 4M: r 3.7: 4 5.49 / 3.96, 8 7.03 / 8.26;   r 7.9: 4 7.95 / 5.36, 8 11.1 / 10.6
+// D2: 7-point mesh (k 7, r 6) 80^3 1.05 / 1.24, 110^3 2.30 / 2.00, 128^3 3.50 / 2.97, 256^3
+// 22.2 / 21.9; 27-point mesh (26, 25) 128^3 13.8 / 22.5; grid (5, 4) 0.5M 0.79 / 0.84, 1M 1.24 /
+// 1.11, 16M 16.0 / 11.4; random, mean degree 8 (9, 9) 0.5M 2.33 / 2.64, 4M 12.7 / 11.7.
+// The line is the least-squares fit (in the logarithm of what the wrong way costs)
+// over 265 such points; one of them loses 9% by it, none else more than 4.5%.  All
+// measured nets fit a warp; a longer one means as many rounds as it has members, and
+// many small rounds are what the lists are for.
 static bool net_rounds_pay(int n, const State& hs) {
-    return n >= 1000000 && hs.max_net <= 32 && hs.members <= 512 &&
-           hs.pairs < (unsigned long long)n * (32u + (unsigned)n / 65536u);
+    if (n < 700000 || hs.max_net > 32 || hs.h_first == 0) return false;
+    const double k = (double)hs.h_first / n, r = (double)hs.pairs / (double)hs.h_first;
+    return k < 3.5 + (0.6 + 0.1 * std::log2(n / 1048576.0)) * r;
 }
 
 // The coloring as a distance-1 coloring of the conflict graph, once net_init
