@@ -17,16 +17,6 @@ __device__ __forceinline__ uint64_t prio_hash(uint64_t seed, uint32_t v) {
     return z ^ (z >> 31);
 }
 
-// True if u has priority over v: key(u) > key(v) with key = (deg, -h, -id).
-// This is Alg. 4 read as one comparison: of two equal-colored vertices the
-// one that does NOT have priority is recolored.
-__device__ __forceinline__ bool has_priority(int du, uint64_t hu, int u,
-                                             int dv, uint64_t hv, int v, bool use_deg) {
-    if (use_deg && du != dv) return du > dv;
-    if (hu != hv) return hu < hv;
-    return u < v;
-}
-
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & (kWarp - 1); }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -34,9 +24,6 @@ __device__ __forceinline__ unsigned long long global_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-
-// Streaming (read-once) 32-bit load for adjacency data.
-__device__ __forceinline__ int ld_stream(const int* p) { return __ldcs(p); }
 
 }  // namespace pgc
 
@@ -97,14 +84,6 @@ __device__ __forceinline__ int warp_max(int x) {
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long x) {
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
     return x;
-}
-
-// Index of the first word of v's forbidden-color bitmap.  Vertex v owns
-// floor(deg(v)/32) + 1 words (bits for colors 1..deg(v)+1, enough because a
-// first-fit color never exceeds deg(v)+1); with offset floor(rp[v]/32) + v
-// consecutive vertices never overlap and the total is nnz/32 + n + 1 words.
-__device__ __forceinline__ long long bitmap_offset(int rp_v, int v) {
-    return (long long)(rp_v >> 5) + v;
 }
 
 }  // namespace pgc
