@@ -187,8 +187,11 @@ pgc_status pgc_color_d1(int32_t n, const int32_t *row_ptr, const int32_t *col_id
  * false): every two vertices joined by a path of one or two edges get
  * different colors.  Arguments, layout and ownership as pgc_color_d1; the
  * priority degree is the row length (1-hop degree).  Colors up to 4096 are
- * supported (PGC_ERR_NO_CONVERGE beyond).  Detection is net based: the
- * closed neighborhood N[u] of every vertex u is a net (Sec. 3.5, NB_BIT).
+ * supported (PGC_ERR_NO_CONVERGE beyond).  The closed neighborhood N[u] of
+ * every vertex u is a net (Sec. 3.5, NB_BIT).  The rounds run over conflict
+ * lists (each vertex's net mates, gathered once) or visit the nets, whichever
+ * is faster for the problem's size and fits the device memory; colors, rounds
+ * and num_colors are the same.  So are those of partial distance 2.
  */
 pgc_status pgc_color_d2(int32_t n, const int32_t *row_ptr, const int32_t *col_idx,
                         uint64_t seed, int32_t *colors, int32_t *rounds,

@@ -94,7 +94,9 @@ struct SingleView {
     // absolute start of v's row from an entry's row start
     __device__ __forceinline__ int begin(int, int r0) const { return r0; }
     using Off = int;
-    // first overflow word of v, whose row starts at b: v owns deg/32 + 1 words
+    // first overflow word of v, whose row starts at b: v owns deg/32 + 1 words (colors
+    // 65 .. deg + 1, the last that first fit can reach), so consecutive vertices never
+    // overlap and the total is nnz/32 + n + 1
     __device__ __forceinline__ long long bm(int v, long long b) const { return (b >> 5) + v; }
     // the degree in v's priority, from its row length d
     __device__ __forceinline__ int degree(int, int d) const { return d; }
@@ -167,16 +169,18 @@ constexpr int kBuildS = 32;     // setup: degree up to this: one thread
 constexpr int kBuildM = 512;    // setup: degree up to this: one warp
 constexpr int kBuildItem = 512; // setup: adjacency items of this length
 constexpr int kPushItem = 128;  // push: adjacency items of this length
-// round-varying priorities: longer lists take a block.  A small graph has few
-// of them and a warp on one is what a round waits for; a large one has enough
-// long lists to fill the grid, and blocks on the shorter of them wait at their
-// barriers.  Dynamic degree, edge factor 16, with blocks from 1024 / 2048 / 4096
-// entries up: R-MAT 18 4.2 / 5.3 / 5.3 ms, R-MAT 20 12.7 / 11.1 / 16.0 ms, R-MAT 21
+// round-varying priorities: longer lists take a block.  With few long lists a
+// warp on one is what a round waits for; with enough of them to fill the grid,
+// blocks on the shorter ones wait at their barriers.  n stands in for their
+// number, which nothing has counted when the line is drawn; measured on R-MAT
+// graphs of edge factor 16 only, where the two grow together.
+// Dynamic degree, with blocks from 1024 / 2048 / 4096 entries up: R-MAT 18 4.2 / 5.3 / 5.3 ms, R-MAT 20 12.7 / 11.1 / 16.0 ms, R-MAT 21
 // 22.0 / 19.0 / 18.9 ms, R-MAT 22 39.3 / 38.6 / 34.0 ms, R-MAT 24 191 / 190 / 152 ms
 // (from 16,384 up: R-MAT 22 55 ms, R-MAT 24 155 ms)
 inline int varying_hub(int n) { return std::clamp(n >> 9, 1024, 4096); }
-// winners up to this degree push inline: 32 / 128 / 512 take 73.7 / 58.5 / 58.5 ms
-// for the 4096-graph batch and 3.68 / 3.66 / 4.05 ms for R-MAT 20
+// winners up to this degree push inline: 32 / 128 / 512 take 58.1 / 46.8 / 46.7 ms
+// for the 4096-graph batch, 3.0 / 3.1 / 3.9 for R-MAT 20, 11.5 / 11.5 / 13.6 for PD2
+// 4M x 1M and 12.8 / 13.7 / 13.7 for the 27-point mesh 128^3 (rows of 124)
 constexpr int kInlinePush = 128;
 
 enum : int {
@@ -322,8 +326,10 @@ __device__ __forceinline__ void block_append(bool a, bool b, int4 e, int4* la, i
     __syncthreads();
 }
 
-// key(u) > key(v) for u, v of the same graph (hash of graph-local ids),
-// hashing only when the degree term does not decide.
+// key(u) > key(v) for u, v of the same graph, key = (deg, -h, -id) (hash of
+// graph-local ids), hashing only when the degree term does not decide.  This is
+// Alg. 4 read as one comparison: of two equal-colored vertices the one that does
+// NOT have priority is recolored.
 __device__ __forceinline__ bool higher(int du, int u, int dv, uint64_t hv, int v, int base,
                                        unsigned long long seed, bool use_deg) {
     if (use_deg && du != dv) return du > dv;
@@ -968,9 +974,9 @@ __global__ void d1_tier(const Problem<V>* __restrict__ Pp, State* st) {
 // the longest list of a warp; with the shared counters read once per block
 // (Hot) and appended to once per block, detection of R-MAT 20's first 13
 // rounds went from 0.86 to 0.57 ms, of PD2 4M x 1M's 51 rounds from 9.6 to
-// 4.6 ms, of the 4096-graph batch from 56 to 32 ms.  64 registers (4 blocks
-// per SM) beat 48 with spills (PD2 16.4 against 16.1 ms, R-MAT 20 3.84
-// against 3.66 ms in all).
+// 4.6 ms, of the 4096-graph batch from 56 to 31 ms.  64 registers (4 blocks
+// per SM) beat 48 with spills (whole colorings: 46.8 against 50.9 ms for the
+// batch, 28.0 against 28.6 for R-MAT 24, 11.5 against 11.7 for PD2 4M x 1M).
 template <bool DYN, class V>
 __device__ __forceinline__ void detect_tier(const Problem<V>& P, const int4* list, int n, int4* next,
                                             int* next_cnt, IdxAppend& app, unsigned char* slot,
@@ -1843,7 +1849,7 @@ __device__ __forceinline__ int pop_bit(uint4& b) {
 //
 // Measured on R-MAT 20 (136 rounds from 3,940 vertices): 2.68 ms for the
 // whole phase as a cooperative launch of 32 blocks over induced lists in L2
-// with three grid barriers per round, 1.06 ms here, of which the loop takes
+// with three grid barriers per round, 0.98 ms here, of which the loop takes
 // 14,300 cycles per round (the two barriers 3,300 with their waiting).  512
 // threads beat 1024 (19,300 cycles: issue slots and block barriers).
 template <class V>

@@ -897,8 +897,10 @@ __global__ void net_commit(const Problem* __restrict__ Pp, cudaGraphConditionalH
 // together (coalesced color gathers in every round).  Rows are handed out from
 // one counter in chunks, in any order.
 //
-// Bound by issue (about 2,500 warp instructions per vertex of the 27-point
-// mesh 128^3, 6.3 ms for its 2.1M vertices; PD2 4M x 1M 4.2 ms).  A hash that
+// The 27-point mesh 128^3 (6.3 ms for its 2.1M vertices) is bound by issue: about
+// 2,500 warp instructions per vertex.  PD2 4M x 1M (4.2 ms) is not: 39% of the
+// issue slots are used by 30% of the warps (ncu, 1M x 256K); it waits for the
+// pattern from DRAM and the members' keys.  A hash that
 // kept blocks of 32 ids together put whole runs of a mesh on top of each
 // other (39 ms); reading the set out slot by slot took 10 ms.
 //
@@ -1067,6 +1069,9 @@ __global__ void __launch_bounds__(256, 4) net_lists(const Problem* __restrict__ 
                         while (log < a.log && (1 << log) < 2 * total) ++log;
                     }
                     members = total;
+                    // (every member has to fit the list, whose bound is the
+                    // problem's largest member count: one vertex above it turns
+                    // the skipping off for all)
                     distinct = few_repeats && (x & 15) != 0 && a.members <= fresh_cap;
                     for (int s = lane; !distinct && s < (1 << log) / 4; s += 32)
                         reinterpret_cast<uint4*>(set)[s] =
