@@ -176,13 +176,28 @@ __global__ void net_init(const Problem* __restrict__ Pp) {
     my_pairs = warp_sum(my_pairs);
     my_members = warp_max(my_members);
     my_net = warp_max(my_net);
+    // a block's together first: six words that every warp of the grid would hit
+    __shared__ int s_max[4];
+    __shared__ unsigned long long s_sum[2];
+    if (threadIdx.x < 4) s_max[threadIdx.x] = 0;
+    if (threadIdx.x < 2) s_sum[threadIdx.x] = 0ull;
+    __syncthreads();
     if (lane_id() == 0) {
-        atomicMax(&st->max_net, my_net);
-        if (my_pairs) atomicAdd(&st->pairs, my_pairs);
-        atomicMax(&st->bound, my_bound);
-        atomicMax(&st->members, my_members);
-        if (P.use_deg) atomicMax(&st->max_deg, my_deg);
-        if (my_h) atomicAdd(&st->h_first, my_h);
+        atomicMax(&s_max[0], my_bound);
+        atomicMax(&s_max[1], my_members);
+        atomicMax(&s_max[2], my_net);
+        atomicMax(&s_max[3], my_deg);
+        atomicAdd(&s_sum[0], my_pairs);
+        atomicAdd(&s_sum[1], my_h);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_sum[1]) {
+        atomicMax(&st->bound, s_max[0]);
+        atomicMax(&st->members, s_max[1]);
+        atomicMax(&st->max_net, s_max[2]);
+        if (P.use_deg) atomicMax(&st->max_deg, s_max[3]);
+        atomicAdd(&st->pairs, s_sum[0]);
+        atomicAdd(&st->h_first, s_sum[1]);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->round = 1;
