@@ -395,10 +395,10 @@ const char *pgc_version(void);
  *   message is "a grid barrier of the mid loop timed out".
  * pgc_test_list_room(limit, buffer): distance-2 and partial distance-2 colorings
  *   over conflict lists: the lists may take at most `limit` entries (0: the
- *   default, 2^29; otherwise this alone decides whether they are built, also
- *   where net rounds would be faster), and their buffer gets at most `buffer`
- *   (0: no limit), so that a build runs out of room.  The problem is then
- *   colored in net rounds, with the same result.
+ *   default, 2^29; 2^31 - 1 at most; otherwise this alone decides whether they
+ *   are built, also where net rounds would be faster), and their buffer gets at
+ *   most `buffer` (0: no limit), so that a build runs out of room.  The problem
+ *   is then colored in net rounds, with the same result.
  */
 pgc_status pgc_test_fail_alloc(int32_t after);
 pgc_status pgc_test_core_barrier(uint32_t polls, int32_t slow_block, uint32_t slow_us);

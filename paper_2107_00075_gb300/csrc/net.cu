@@ -1451,7 +1451,9 @@ static pgc_status run_lists(Context& cx, const Input& in, int nnz, const State& 
     E* eng = d1::engine_for<d1::ListView>(cx.dev.device);
     std::lock_guard<std::mutex> lk(eng->mu);
     eng->dev = cx.dev;
-    const unsigned long long limit = th.list_limit ? th.list_limit : kListMaxEntries;
+    // (a row's first entry is an int)
+    const unsigned long long limit =
+        th.list_limit ? std::min<unsigned long long>(th.list_limit, INT32_MAX) : kListMaxEntries;
 
     ListArgs a = {};
     a.log = kListMinLog;
